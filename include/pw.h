@@ -99,7 +99,8 @@ typedef void *pw_stream_t; /* cudaStream_t */
  * 128-byte boundary, pitch_j a multiple of 128 bytes.  Writes the grid to
  * *out and the number of elements each field allocation must hold to
  * *alloc_elems (may be NULL).  This layout qualifies for the TMA k-march
- * kernel when nx is a multiple of 4.
+ * kernel when nx is a multiple of 4; other widths from 32 up take that kernel
+ * too once the grid holds 2^19 cells (see pw_set_kernel).
  */
 pw_status_t pw_grid_default(int32_t nx, int32_t ny, int32_t nz, int32_t halo, pw_dtype_t dtype,
                             pw_grid_t *out, int64_t *alloc_elems);
@@ -126,7 +127,10 @@ pw_status_t pw_destroy(pw_handle_t h);
 
 /* Kernel selection for pw_tendencies, pw_step, pw_step_to and the periodic
  * pw_adjoint: 0 = automatic (TMA k-march kernel when the layout and pointers
- * qualify, else the generic kernel), 1 = generic kernel, 2 = TMA kernel
+ * qualify, else the generic kernel; a width that is no multiple of 4 qualifies
+ * for pw_tendencies and the step calls when no launch shape was fixed, nx >= 32
+ * and the grid has at least 2^19 cells), 1 = generic kernel, 2 = TMA kernel,
+ * for widths that are a multiple of 4
  * (pw_tendencies and the step calls return PW_ERR_UNSUPPORTED/PW_ERR_ALIGN
  * when the layout or pointers do not qualify; pw_adjoint then runs the
  * generic kernel). */

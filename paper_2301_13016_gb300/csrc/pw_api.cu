@@ -141,10 +141,10 @@ pw_status_t pw::validate_grid(const pw_grid_t* g) {
 
 // TMA eligibility of the layout (pointer alignment is checked per call).
 // Writes the x offset `ox` of element i = 0 within its padded row.
-bool pw::tma_layout_ok(const pw_grid_t& g, int* ox_out, const char** why) {
+bool pw::tma_layout_ok(const pw_grid_t& g, int* ox_out, const char** why, bool any_nx) {
     const long long es = (long long)dtype_size(g.dtype);
     const long long padx = 16 / es;
-    if (g.nx % 4) { *why = "nx is not a multiple of 4"; return false; }
+    if (!any_nx && g.nx % 4) { *why = "nx is not a multiple of 4"; return false; }
     if ((g.pitch_j * es) % 16 || (g.pitch_k * es) % 16) { *why = "pitches are not multiples of 16 bytes"; return false; }
     const long long r = g.origin - (long long)(g.halo - 1) * g.pitch_j;
     if (r < 0 || r >= g.pitch_j) { *why = "origin is not within the first padded row"; return false; }
@@ -208,7 +208,8 @@ pw_status_t pw::encode_tensor_map_box(const pw_grid_t& g, const void* ptr, int b
     if (inject_failure(INJECT_TENSOR_MAP)) return fail(PW_ERR_CUDA, "cuTensorMapEncodeTiled failed (injected)");
     int ox = 0;
     const char* why = "";
-    if (!tma_layout_ok(g, &ox, &why)) return fail(PW_ERR_UNSUPPORTED, "layout not TMA-eligible: %s", why);
+    // (the callers decide about widths: a box may run past the row's end)
+    if (!tma_layout_ok(g, &ox, &why, true)) return fail(PW_ERR_UNSUPPORTED, "layout not TMA-eligible: %s", why);
     const size_t es = dtype_size(g.dtype);
     CUtensorMapDataType dt = g.dtype == PW_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                              : g.dtype == PW_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
@@ -273,6 +274,7 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
         }
     } else {
         const bool half = dtype_size(gr.dtype) == 2;
+        c.rag = gr.nx % 4 != 0;
         c.lx = 32;
         c.nc = 4;
         c.ty = 4;
@@ -280,7 +282,7 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
         c.rp = 1;
         if (gr.nx <= 64) {
             c.lx = 16;
-        } else if (half && (!step || gr.nx % 8 == 0)) {
+        } else if (half && (!step || gr.nx % 8 == 0 || c.rag)) {
             c.lx = 16;   // x pairs of 8 cells: tiles of 128 columns
             c.nc = 8;
             c.ty = 8;
@@ -322,6 +324,35 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
     if (c.nseg > gr.nz / 2) c.nseg = std::max(1, gr.nz / 2);
     cache = c;
     return c;
+}
+
+// TMA k-march or generic kernel for the source terms and the steps: what
+// pw_set_kernel asked for, else TMA when the layout and every pointer qualify.
+// A width that is no multiple of 4 takes the k-march too (its RAG kernels) when
+// the shape is automatic and the grid has at least kRagMinCells cells:
+// measured on GB300, FP32 source terms, generic against k-march: 191x64x32
+// 5.7 / 6.0 us, 255x64x32 6.8 / 5.7, 63x256x64 11.3 / 8.2, 511x256x64 112 / 46,
+// 1021x1023x61 943 / 266.  A width below kRagMinNx would leave more than half
+// of the narrowest tile (64 columns) idle.  pw_set_kernel(2) refuses such a
+// width as it always has.
+constexpr int kRagMinNx = 32;
+constexpr long long kRagMinCells = 1 << 19;
+static pw_status_t march_kernel_choice(pw_handle_t h, const void* const* bufs, int n, bool* use_tma, int* ox) {
+    const char* why = "";
+    const TmaConfig& u = h->tma_user;
+    const pw_grid_t& gr = h->grid;
+    const bool any_nx = h->kernel_kind == 0 && gr.nx >= kRagMinNx &&
+                        (long long)gr.nx * gr.ny * gr.nz >= kRagMinCells &&
+                        !(u.lx || u.nc || u.ty || u.stages || u.rp);
+    const bool layout_ok = tma_layout_ok(h->grid, ox, &why, any_nx);
+    bool ptrs_ok = true;
+    for (int a = 0; a < n; ++a) ptrs_ok = ptrs_ok && aligned16(bufs[a]);
+    if (h->kernel_kind == 2) {
+        if (!layout_ok) return fail(PW_ERR_UNSUPPORTED, "TMA kernel requested but %s", why);
+        if (!ptrs_ok) return fail(PW_ERR_ALIGN, "TMA kernel requested but a field pointer is not 16-byte aligned");
+    }
+    *use_tma = (h->kernel_kind == 2) || (h->kernel_kind == 0 && layout_ok && ptrs_ok);
+    return PW_OK;
 }
 
 static void make_scales(const float* scale, Scales* sc, bool* scaled) {
@@ -632,8 +663,8 @@ pw_status_t pw_tendencies(pw_handle_t h, const void* u, const void* v, const voi
             if (o == i) return fail(PW_ERR_ARG, "an output aliases an input");
     if (su == sv || su == sw || sv == sw) return fail(PW_ERR_ARG, "outputs alias each other");
     {
-        const void* all[6] = {u, v, w, su, sv, sw};
-        pw_status_t dst = check_device_ptrs(h, all, 6);
+        const void* ptrs[6] = {u, v, w, su, sv, sw};
+        pw_status_t dst = check_device_ptrs(h, ptrs, 6);
         if (dst != PW_OK) return dst;
     }
     if (scale)
@@ -647,16 +678,10 @@ pw_status_t pw_tendencies(pw_handle_t h, const void* u, const void* v, const voi
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
     int ox = 0;
-    const char* why = "";
-    bool layout_ok = tma_layout_ok(h->grid, &ox, &why);
-    bool ptrs_ok = true;
-    for (auto p : ins) ptrs_ok = ptrs_ok && aligned16(p);
-    for (auto p : outs) ptrs_ok = ptrs_ok && aligned16(p);
-    bool use_tma = (h->kernel_kind == 2) || (h->kernel_kind == 0 && layout_ok && ptrs_ok);
-    if (h->kernel_kind == 2) {
-        if (!layout_ok) return fail(PW_ERR_UNSUPPORTED, "TMA kernel requested but %s", why);
-        if (!ptrs_ok) return fail(PW_ERR_ALIGN, "TMA kernel requested but a field pointer is not 16-byte aligned");
-    }
+    const void* all[6] = {u, v, w, su, sv, sw};
+    bool use_tma = false;
+    pw_status_t kst = march_kernel_choice(h, all, 6, &use_tma, &ox);
+    if (kst != PW_OK) return kst;
     if (use_tma) {
         TmaConfig c = choose_tma(h, false);
         CUtensorMap maps[3];
@@ -881,21 +906,6 @@ static pw_status_t step_pass(pw_handle_t h, const GridDev& g, const void* const*
     return PW_OK;
 }
 
-// TMA or generic for the step entry points: what pw_set_kernel asked for,
-// else TMA when the layout and every pointer qualify.
-static pw_status_t step_kernel_choice(pw_handle_t h, void* const* bufs, int n, bool* use_tma, int* ox) {
-    const char* why = "";
-    const bool layout_ok = tma_layout_ok(h->grid, ox, &why);
-    bool ptrs_ok = true;
-    for (int a = 0; a < n; ++a) ptrs_ok = ptrs_ok && aligned16(bufs[a]);
-    if (h->kernel_kind == 2) {
-        if (!layout_ok) return fail(PW_ERR_UNSUPPORTED, "TMA kernel requested but %s", why);
-        if (!ptrs_ok) return fail(PW_ERR_ALIGN, "TMA kernel requested but a field pointer is not 16-byte aligned");
-    }
-    *use_tma = (h->kernel_kind == 2) || (h->kernel_kind == 0 && layout_ok && ptrs_ok);
-    return PW_OK;
-}
-
 pw_status_t pw_step_to(pw_handle_t h, const void* u, const void* v, const void* w, void* nu, void* nv, void* nw,
                        float dt, const float* scale, pw_stream_t stream) {
     PW_RANGE("pw_step_to");
@@ -915,13 +925,13 @@ pw_status_t pw_step_to(pw_handle_t h, const void* u, const void* v, const void* 
     if (st != PW_OK) return st;
     bool use_tma = false;
     int ox = 0;
-    st = step_kernel_choice(h, bufs, 6, &use_tma, &ox);
+    st = march_kernel_choice(h, bufs, 6, &use_tma, &ox);
     if (st != PW_OK) return st;
     const GridDev g = to_dev(h->grid);
     CoefDev cf{h->tcx, h->tcy, h->d_tz};
     TmaConfig c{};
     if (use_tma) c = choose_tma(h, true);
-    if (use_tma && h->grid.nx % c.nc)
+    if (use_tma && !c.rag && h->grid.nx % c.nc)
         return fail(PW_ERR_UNSUPPORTED, "fused steps with cells=%d need nx to be a multiple of %d", c.nc, c.nc);
     st = step_pass(h, g, bufs, bufs + 3, sc, scaled, cf, dt, use_tma, ox, c, reinterpret_cast<cudaStream_t>(stream));
     if (st != PW_OK) return st;
@@ -957,12 +967,12 @@ pw_status_t pw_step(pw_handle_t h, void* u, void* v, void* w, void* tmp_u, void*
     }
     int ox = 0;
     bool use_tma = false;
-    sst = step_kernel_choice(h, bufs, 6, &use_tma, &ox);
+    sst = march_kernel_choice(h, bufs, 6, &use_tma, &ox);
     if (sst != PW_OK) return sst;
     // two steps per pass: TMA path, a lateral halo >= 2, and interior rows
     // starting at least 7 elements into their padded row (the q0 box begins
     // 7 columns before the first interior column)
-    const bool tb2_ok = use_tma && g.halo >= 2 && ox >= 7;
+    const bool tb2_ok = use_tma && g.nx % 4 == 0 && g.halo >= 2 && ox >= 7;
     if (h->steps_per_pass == 2 && nsteps >= 2 && !tb2_ok)
         return fail(PW_ERR_UNSUPPORTED, "two steps per pass need the TMA path, a halo >= 2 and >= 7 columns before "
                                         "the interior in each padded row");
@@ -971,7 +981,7 @@ pw_status_t pw_step(pw_handle_t h, void* u, void* v, void* w, void* tmp_u, void*
     const bool use_tb2 = tb2_ok && h->steps_per_pass == 2;
     TmaConfig c{};
     if (use_tma) c = choose_tma(h, true);
-    if (use_tma && h->grid.nx % c.nc)
+    if (use_tma && !c.rag && h->grid.nx % c.nc)
         return fail(PW_ERR_UNSUPPORTED, "fused steps with cells=%d need nx to be a multiple of %d", c.nc, c.nc);
     Step2Config c2{};
     if (use_tb2 && nsteps >= 2) c2 = choose_step2(h);

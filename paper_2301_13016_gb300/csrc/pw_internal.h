@@ -112,6 +112,7 @@ struct TmaConfig {
     int seg_count = 0;  // segments to launch (0 = all nseg)
     int rp = 1;         // rows per thread: 1, or 2 (packed FP32x2 arithmetic on row pairs)
     int xp = 0;         // 1: one row per thread, its nc cells packed as FP32x2 pairs (cell q, cell q + nc/2)
+    int rag = 0;        // 1: nx is no multiple of 4 (a row's last vector may hold 1 to nc cells)
 };
 
 // Launch shape of the two-step (temporal blocking) k-march kernel.
@@ -231,7 +232,8 @@ pw_status_t internal_check_device_ptrs(pw_handle_t h, const void* const* ps, int
 
 // Layout checks and TMA descriptors shared by the single-grid and batched paths.
 pw_status_t validate_grid(const pw_grid_t* g);
-bool tma_layout_ok(const pw_grid_t& g, int* ox_out, const char** why);
+// any_nx: accept an nx that is no multiple of 4 (the RAG kernels)
+bool tma_layout_ok(const pw_grid_t& g, int* ox_out, const char** why, bool any_nx = false);
 bool aligned16(const void* p);
 // p is device (or managed) memory of the given GPU.
 bool is_device_ptr(const void* p, int device);

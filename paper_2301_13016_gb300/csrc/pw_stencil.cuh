@@ -51,6 +51,21 @@ struct Epilogue<T, MODE_TEND> {
                                                        int, int* err = nullptr) {
         if (dbg_store(g, o, N, true, err)) storev<N>(of + o, a);
     }
+    // the first nv < N cells of a row vector that runs past nx
+    template <int N>
+    static __device__ __forceinline__ void store_tail(T* of, long long o, const float (&a)[N], const int nv,
+                                                      const GridDev& g, int, int, int* err = nullptr) {
+        if constexpr (N == 8) {   // half a vector where it fits
+            if (nv >= 4) {
+                const float h4[4] = {a[0], a[1], a[2], a[3]};
+                if (dbg_store(g, o, 4, true, err)) storev<4>(of + o, h4);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < N - 1; ++q)
+            if (q < nv && (q >= 4 || nv < 4 || N == 4) && dbg_store(g, o + q, 1, true, err))
+                of[o + q] = Store<T>::from_f(a[q]);
+    }
 };
 
 // Periodic images of a step's output cells in a lateral halo of any depth
@@ -148,6 +163,32 @@ struct Epilogue<T, MODE_STEP> {
                 of[p + g.nx] = Store<T>::from_f(a[0]);                  // cell i = 1 -> i = nx+1
             if (east && dbg_store(g, p + (N - 1) - g.nx, 1, false, err))
                 of[p + (N - 1) - g.nx] = Store<T>::from_f(a[N - 1]);    // cell i = nx -> i = 0
+        }
+    }
+    // the first nv < N cells (j, i0..nx) of a row vector that runs past nx: the
+    // last of them is cell nx, the first may be cell 1 too
+    template <int N>
+    static __device__ __forceinline__ void store_tail(T* of, long long o, const float (&a)[N], const int nv,
+                                                      const GridDev& g, int j, int i0, int* err = nullptr) {
+        const bool img = g.halo == 1;   // deeper halos are refreshed by the halo kernel
+        const long long dyp = (img && j == 1) ? (long long)g.ny * g.pj : 0;
+        const long long dym = (img && j == g.ny) ? -(long long)g.ny * g.pj : 0;
+        const long long shifts[3] = {0, dyp, dym};
+        T t[N];
+#pragma unroll
+        for (int q = 0; q < N; ++q) t[q] = Store<T>::from_f(a[q]);
+        T last = t[0];   // cell nx
+#pragma unroll
+        for (int q = 1; q < N - 1; ++q) last = (q == nv - 1) ? t[q] : last;
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            if (s > 0 && shifts[s] == 0) continue;
+            const long long p = o + shifts[s];
+#pragma unroll
+            for (int q = 0; q < N - 1; ++q)
+                if (q < nv && dbg_store(g, p + q, 1, s == 0, err)) of[p + q] = t[q];
+            if (img && i0 == 1 && dbg_store(g, p + g.nx, 1, false, err)) of[p + g.nx] = t[0];
+            if (img && dbg_store(g, p + (nv - 1) - g.nx, 1, false, err)) of[p + (nv - 1) - g.nx] = last;
         }
     }
 };
@@ -880,7 +921,10 @@ __device__ __forceinline__ void load_pairs_sa(uint32_t a, float2 (&o)[NC / 2]) {
 // packed as NC/2 pairs (cell q, cell q + NC/2), so that a staged row unpacks
 // straight into FP32x2 operands and the x neighbours beyond the vector come
 // from the staged row itself.
-template <typename T, int LX, int TY, int S, int MODE, int NC = 4, int RP = 1, int XP = 0>
+// RAG = 1: any nx; a row's last vector may hold 1 to NC cells of the grid
+// (store_tail).  Its other cells are computed from the halo column, the rest
+// of the padded row or the tensor map's zero fill, and not stored.
+template <typename T, int LX, int TY, int S, int MODE, int NC = 4, int RP = 1, int XP = 0, int RAG = 0>
 __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP, XP>& sm, const CUtensorMap* tm_u,
                                            const CUtensorMap* tm_v, const CUtensorMap* tm_w, T* __restrict__ o0,
                                            T* __restrict__ o1, T* __restrict__ o2, const GridDev& g, const int ox,
@@ -1056,7 +1100,12 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
                         a[c] = MODE == MODE_STEP ? fmaf(dt, cellv(rr, c, half), cellv(q, c, half))
                                                  : cellv(rr, c, half);
                     const long long o = row_off + (long long)half * g.pj + (long long)kk * g.pk;
-                    if constexpr (MODE == MODE_TEND && NC == 8) {
+                    if constexpr (RAG) {
+                        if (i0 + NC - 1 > g.nx) {
+                            Epilogue<T, MODE>::template store_tail<NC>(of, o, a, g.nx - i0 + 1, g, j + half, i0, err);
+                            return;
+                        }
+                    } else if constexpr (MODE == MODE_TEND && NC == 8) {
                         // nx = 4 mod 8: the row's last vector holds 4 cells of
                         // the grid (the other 4 were computed from halo and
                         // padding columns and are not stored)
@@ -1203,7 +1252,7 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
 }
 
 // One grid, one tile per CTA: blockIdx = (tile column, tile row, k segment).
-template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP>
+template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP, int RAG>
 __global__ void __launch_bounds__(TmaLayout<T, LX, TY, S, NC, RP, XP>::THREADS,
                                   (tma_min_blocks<T, LX, TY, S, NC, RP, XP>()))
     tma_kernel(const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_v,
@@ -1218,7 +1267,7 @@ __global__ void __launch_bounds__(TmaLayout<T, LX, TY, S, NC, RP, XP>::THREADS,
     if (ke < kb) return;   // empty k segment (the host never launches one)
     sm.init(threadIdx.y * 32 + threadIdx.x);
     uint32_t ring = 0;
-    march_tile<T, LX, TY, S, MODE, NC, RP, XP>(sm, &tm_u, &tm_v, &tm_w, o0, o1, o2, g, ox, kc, dt, blockIdx.x,
+    march_tile<T, LX, TY, S, MODE, NC, RP, XP, RAG>(sm, &tm_u, &tm_v, &tm_w, o0, o1, o2, g, ox, kc, dt, blockIdx.x,
                                                blockIdx.y, kb, ke, ring, err);
 }
 
@@ -1235,10 +1284,14 @@ __global__ void __launch_bounds__(TmaLayout<T, LX, TY, S, NC, RP, XP>::THREADS,
     X(16, 8, 4, 4, 1, 1) X(8, 8, 4, 8, 1, 1) X(8, 16, 4, 8, 1, 1) X(8, 16, 4, 4, 1, 0) X(32, 16, 4, 4, 1, 0)      \
     X(16, 16, 4, 4, 1, 0)
 
+// Shapes for a width that is no multiple of 4 (RAG kernels): the automatic
+// ones only; a shape the caller fixed keeps to the generic kernel there.
+#define PW_TMA_RAGGED(X) X(32, 4, 4, 4, 1, 0) X(16, 4, 4, 4, 1, 0) X(16, 8, 4, 8, 1, 1)
+
 template <typename T, int NC, int RP, int XP = 0>
 constexpr bool nc_ok() { return (NC == 4 && RP == 1 && XP == 0) || sizeof(T) == 2; }
 
-template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP>
+template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP, int RAG = 0>
 static cudaError_t launch_tma_inst(const GridDev& g, int ox, const CUtensorMap* maps, void* o0, void* o1,
                                    void* o2, const Scales& sc, const CoefDev& cf, float dt, int* err, int nseg,
                                    int seg0, int seg_count, cudaStream_t s) {
@@ -1246,7 +1299,7 @@ static cudaError_t launch_tma_inst(const GridDev& g, int ox, const CUtensorMap* 
     return cudaErrorInvalidConfiguration;
   } else {
     using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
-    auto kern = tma_kernel<T, LX, TY, S, MODE, NC, RP, XP>;
+    auto kern = tma_kernel<T, LX, TY, S, MODE, NC, RP, XP, RAG>;
     cudaError_t e = set_smem_attr_once(kern, (int)L::SMEM);
     if (e != cudaSuccess) return e;
     if (seg_count <= 0) seg_count = nseg - seg0;
@@ -1266,6 +1319,15 @@ static cudaError_t launch_tma_mode(const GridDev& g, int ox, const CUtensorMap* 
     if (c.lx == LX_ && c.ty == TY_ && c.stages == S_ && c.nc == NC_ && c.rp == RP_ && c.xp == XP_)      \
         return launch_tma_inst<T, LX_, TY_, S_, MODE, NC_, RP_, XP_>(g, ox, maps, o0, o1, o2, sc, cf, dt, err, \
                                                                      c.nseg, c.seg0, c.seg_count, s);
+    if (c.rag) {
+#define PW_DISPATCH_RAG(LX_, TY_, S_, NC_, RP_, XP_)                                                        \
+    if (c.lx == LX_ && c.ty == TY_ && c.stages == S_ && c.nc == NC_ && c.rp == RP_ && c.xp == XP_)          \
+        return launch_tma_inst<T, LX_, TY_, S_, MODE, NC_, RP_, XP_, 1>(g, ox, maps, o0, o1, o2, sc, cf, dt, err, \
+                                                                        c.nseg, c.seg0, c.seg_count, s);
+        PW_TMA_RAGGED(PW_DISPATCH_RAG)
+#undef PW_DISPATCH_RAG
+        return cudaErrorInvalidConfiguration;
+    }
     PW_TMA_CONFIGS(PW_DISPATCH)
 #undef PW_DISPATCH
     return cudaErrorInvalidConfiguration;
