@@ -296,7 +296,7 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
     } else {
         const long long tiles =
             (long long)((gr.nx + c.nc * c.lx - 1) / (c.nc * c.lx)) * ((gr.ny + c.ty - 1) / c.ty);
-        int bps = tma_blocks_per_sm(gr.dtype, c);
+        int bps = step ? step_blocks_per_sm(gr.dtype, c) : tma_blocks_per_sm(gr.dtype, c);
         if (bps < 1) bps = 1;
         const long long slots = (long long)h->num_sms * bps;
         // the count that minimises (waves of CTAs) x (planes each CTA marches:

@@ -50,7 +50,7 @@ struct BatchShapes {
     static constexpr int MAPS = DUAL ? 6 : 3;   // tensor maps per grid (u, v, w per shape)
     static_assert(!DUAL || LN::THREADS == LW::THREADS, "both shapes use every thread of the CTA");
     static_assert(!DUAL || 2 * LN::TX == LW::TX, "the narrow shape is half as wide");
-    static_assert(LN::CTAB == LW::CTAB, "one coefficient-table layout");
+    static_assert(LN::PACKED == LW::PACKED, "one coefficient-table layout");
 };
 
 // Resident CTAs per SM the batch kernel's register budget is sized for (at

@@ -180,7 +180,8 @@ AdjConfig adjoint_default_config();
 int adjoint_blocks_per_sm(const AdjConfig& c);
 
 // Blocks of the TMA kernel resident per SM for a config (0 if it cannot launch).
-int tma_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c);
+int tma_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c);    // source terms
+int step_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c);   // fused steps
 
 cudaError_t launch_fill_halo(pw_dtype_t dt, const GridDev& g, void* f, int num_sms, cudaStream_t s);
 

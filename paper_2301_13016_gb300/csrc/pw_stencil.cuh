@@ -46,7 +46,7 @@ struct Epilogue<T, MODE_TEND> {
         o2[o] = Store<T>::from_f(c);
     }
     // one field's row vector of N cells
-    template <int N>
+    template <int N, bool>
     static __device__ __forceinline__ void store_field(T* of, long long o, const float (&a)[N], const GridDev& g, int,
                                                        int, int* err = nullptr) {
         if (dbg_store(g, o, N, true, err)) storev<N>(of + o, a);
@@ -142,27 +142,36 @@ struct Epilogue<T, MODE_STEP> {
         o2[o] = tc;
         StepImages::cell<T>(o0, o1, o2, o, ta, tb, tc, g, j, i);
     }
-    // one field's vector of N cells (j, i0..i0+N-1), i0 = 1 mod N, nx = 0 mod N
-    template <int N>
+    // one field's vector of N cells (j, i0..i0+N-1), i0 = 1 mod N, nx = 0 mod N.
+    // ONE_TEST (the x-pair forms): one branch decides whether the vector
+    // touches any boundary; without it (scalar FP32) the two column images are
+    // single predicated stores and only the row images sit behind a branch.
+    // Fused step at 2048^2 x 64, us a pass: BF16 745 with ONE_TEST, 793
+    // without; FP32 1092 with, 1011 without.
+    template <int N, bool ONE_TEST>
     static __device__ __forceinline__ void store_field(T* of, long long o, const float (&a)[N], const GridDev& g,
                                                        int j, int i0, int* err = nullptr) {
         if (dbg_store(g, o, N, true, err)) storev<N>(of + o, a);
         if (g.halo != 1) return;   // deeper halos are refreshed by the halo kernel
         const bool west = (i0 == 1), east = (i0 + N - 1 == g.nx);
-        // most row vectors touch no boundary: one test, the same at every level
-        if (!(west | east | (j == 1) | (j == g.ny))) return;
-        const long long dyp = (j == 1) ? (long long)g.ny * g.pj : 0;
-        const long long dym = (j == g.ny) ? -(long long)g.ny * g.pj : 0;
-        const long long shifts[3] = {0, dyp, dym};
+        if (ONE_TEST && !(west | east | (j == 1) | (j == g.ny))) return;
+        // the images of cells 1 and nx of the row at offset p
+        auto columns = [&](const long long p) {
+            if (west && dbg_store(g, p + g.nx, 1, false, err)) of[p + g.nx] = Store<T>::from_f(a[0]);
+            if (east && dbg_store(g, p + (N - 1) - g.nx, 1, false, err))
+                of[p + (N - 1) - g.nx] = Store<T>::from_f(a[N - 1]);
+        };
+        if (!ONE_TEST) {
+            columns(o);
+            if (j != 1 && j != g.ny) return;
+        }
+        const long long shifts[3] = {0, (j == 1) ? (long long)g.ny * g.pj : 0, (j == g.ny) ? -(long long)g.ny * g.pj : 0};
 #pragma unroll
-        for (int s = 0; s < 3; ++s) {
+        for (int s = ONE_TEST ? 0 : 1; s < 3; ++s) {
             if (s > 0 && shifts[s] == 0) continue;
             const long long p = o + shifts[s];
             if (s > 0 && dbg_store(g, p, N, false, err)) storev<N>(of + p, a);   // the row image
-            if (west && dbg_store(g, p + g.nx, 1, false, err))
-                of[p + g.nx] = Store<T>::from_f(a[0]);                  // cell i = 1 -> i = nx+1
-            if (east && dbg_store(g, p + (N - 1) - g.nx, 1, false, err))
-                of[p + (N - 1) - g.nx] = Store<T>::from_f(a[N - 1]);    // cell i = nx -> i = 0
+            columns(p);
         }
     }
     // the first nv < N cells (j, i0..nx) of a row vector that runs past nx: the
@@ -349,6 +358,35 @@ struct NbrShfl {
     }
 };
 
+// Scalar form: shuffles, and the row's edge lanes alone load the value beside
+// their vector from the staged row (ld(f, up, dr, side): side 0 at x = -1,
+// side 1 at x = NC); or (NbrLd) every lane loads it.  On GB300 the shuffles are
+// the faster for the source terms (2048^2 x 64: 977 against 990 us), the loads
+// for the fused step (1011 against 1023; 512^2 x 64 76.4 against 78.7).
+template <int NC, int LX, typename V, class Ld>
+struct NbrShflEdge {
+    const Ld& ld;
+    const int xl;
+    __device__ __forceinline__ V m(int f, int up, int dr, const V (&x)[NC]) const {
+        V s = VOps<V>::shfl_up(x[NC - 1], LX);
+        if (xl == 0) s = ld(f, up, dr, 0);
+        return s;
+    }
+    __device__ __forceinline__ V p(int f, int up, int dr, const V (&x)[NC]) const {
+        V s = VOps<V>::shfl_down(x[0], LX);
+        if (xl == LX - 1) s = ld(f, up, dr, 1);
+        return s;
+    }
+};
+
+template <int NC, typename V, class Ld>
+struct NbrLd {
+    const Ld& ld;
+    const int xl;
+    __device__ __forceinline__ V m(int f, int up, int dr, const V (&)[NC]) const { return ld(f, up, dr, 0); }
+    __device__ __forceinline__ V p(int f, int up, int dr, const V (&)[NC]) const { return ld(f, up, dr, 1); }
+};
+
 // x neighbours when a thread's 2*NP consecutive cells are packed as NP pairs
 // (cell q, cell q + NP): the pair one cell to the left of pair 0 is
 // (x = -1, cell NP - 1) and the pair one to the right of pair NP-1 is
@@ -390,6 +428,26 @@ struct ZCoefLdg {
         ntz2v = VOps<V>::splat(-(t2 * k.kz[1]));
         td1w = VOps<V>::splat(d1 * k.kz[2]);
         ntd2w = VOps<V>::splat(-(d2 * k.kz[2]));
+    }
+};
+
+// The table of the scalar forms: 2 float4 per level, {tz1u, tz1v, ntz2u,
+// ntz2v} and {td1w, ntd2w, -, -}.
+struct ZCoefTab1 {
+    const float4* tab;
+    int base;
+    __device__ __forceinline__ void lower(int kk, float& tz1u, float& tz1v) const {
+        const float2 a = *reinterpret_cast<const float2*>(tab + 2 * (kk - base));
+        tz1u = a.x;
+        tz1v = a.y;
+    }
+    __device__ __forceinline__ void upper(int kk, float& ntz2u, float& ntz2v, float& td1w, float& ntd2w) const {
+        const float2 a = reinterpret_cast<const float2*>(tab + 2 * (kk - base))[1];
+        const float2 b = reinterpret_cast<const float2*>(tab + 2 * (kk - base))[2];
+        ntz2u = a.x;
+        ntz2v = a.y;
+        td1w = b.x;
+        ntd2w = b.y;
     }
 };
 
@@ -436,6 +494,17 @@ __device__ __forceinline__ void zcoef_fill(float4* tab, const FoldedCoef& k, con
             b = -(d2 * k.kz[2]);
         }
         tab[e] = make_float4(a, a, b, b);
+    }
+}
+
+__device__ __forceinline__ void zcoef_fill1(float4* tab, const FoldedCoef& k, const int nzp2, const int lo,
+                                            const int hi, const int tid, const int nthreads) {
+    for (int e = tid; e <= hi - lo; e += nthreads) {
+        const int kk = lo + e;
+        const float t1 = __ldg(k.tz + kk), t2 = __ldg(k.tz + nzp2 + kk);
+        const float d1 = __ldg(k.tz + 2 * nzp2 + kk), d2 = __ldg(k.tz + 3 * nzp2 + kk);
+        tab[2 * e] = make_float4(t1 * k.kz[0], t1 * k.kz[1], -(t2 * k.kz[0]), -(t2 * k.kz[1]));
+        tab[2 * e + 1] = make_float4(d1 * k.kz[2], -(d2 * k.kz[2]), 0.f, 0.f);
     }
 }
 
@@ -700,13 +769,21 @@ __device__ __forceinline__ void march_level(MarchRegs<NC, V>& st, const Row& row
 // Ring bookkeeping is global to the CTA: the n-th plane a CTA ever issues
 // goes to slot n % S and completes phase (n / S) & 1 of that slot's mbarrier,
 // so a persistent CTA can march tile after tile without re-initialising.
-// Build-time knob of the k-march kernel: PW_TMA_MAX_MINB caps the resident
-// CTAs per SM the register budget of the 4-cell shapes is sized for.  On
-// GB300 a cap of 2 (the compiler's own choice, about 128 registers) was the
-// fastest for every 4-cell shape; caps of 4 to 6 made them slower, and the
-// 8-row ones spill.
+// Build-time knobs of the k-march kernel.  PW_TMA_MAX_MINB caps the resident
+// CTAs per SM the register budget of the 4-cell source-term shapes is sized
+// for: 2 leaves the compiler its choice (113 registers, 4 CTAs of 4 warps per
+// SM).  Five CTAs (102 registers, no spills) are faster below about 512^2 x 64
+// (73 -> 71 us) and slower above (2048^2 x 64: 977 -> 1055 us; the same kernel
+// held to 4 resident CTAs takes 983, so it is the memory side that minds).
+// PW_STEP_REGS is the register target of the 4-cell scalar steps: five CTAs
+// per SM there (512^2 / 1024^2 / 2048^2 x 64 FP32: 81 / 288 / 1089 -> 77 / 277 /
+// 1008 us a step); their ragged form keeps the compiler's choice (304 against
+// 345 us at 1021 x 1023 x 61).
 #ifndef PW_TMA_MAX_MINB
 #define PW_TMA_MAX_MINB 2
+#endif
+#ifndef PW_STEP_REGS
+#define PW_STEP_REGS 102
 #endif
 // Register target of the 8-cells-a-thread shapes (8 x 1 or 4 x 2).
 #ifndef PW_TMA_REGS8
@@ -722,7 +799,8 @@ __device__ __forceinline__ void march_level(MarchRegs<NC, V>& st, const Row& row
 #define PW_MARCH_SPLIT_ARRIVE 0
 #endif
 // Levels per iteration of the k-march loop (2: the carried rows of one level
-// are renamed rather than moved into place for the next).
+// are renamed rather than moved into place for the next; x-pair forms only:
+// the scalar march gains nothing, 64^3 loses 4 %).
 #ifndef PW_MARCH_UNROLL
 #define PW_MARCH_UNROLL 1
 #endif
@@ -773,9 +851,9 @@ struct TmaLayout {
     // packed FP32x2 forms read the per-level vertical coefficients from a
     // table in shared memory (ZCoefTab), CTAB_LEVELS levels at a time
     static constexpr bool PACKED = (RP == 2 || XP == 1);
-    static constexpr bool CTAB = PACKED;
-    static constexpr int CTAB_LEVELS = 128;
-    static constexpr size_t CTAB_BYTES = CTAB ? (size_t)CTAB_LEVELS * 3 * sizeof(float4) : 0;
+    static constexpr int CTAB_LEVELS = PACKED ? 128 : 64;
+    static constexpr int CTAB_F4 = PACKED ? 3 : 2;   // float4 per level
+    static constexpr size_t CTAB_BYTES = (size_t)CTAB_LEVELS * CTAB_F4 * sizeof(float4);
     // x-pair form with PW_MARCH_PD_SMEM: the lower flux products of every
     // thread (3 fields x NC/2 pairs) in shared memory between levels
     static constexpr bool PD_SMEM = XP == 1 && PW_MARCH_PD_SMEM;
@@ -806,14 +884,17 @@ struct TmaLayout {
 // measured best on GB300 (16 lanes x 8 cells x 4 rows: 269 -> 295 Gcell/s for
 // BF16 against the compiler's 210 registers, as more CTAs per SM hide more
 // latency; 128 spills and 200 leaves 2 CTAs per SM, both slower).
-template <typename T, int LX, int TY, int S, int NC = 4, int RP = 1, int XP = 0>
+template <typename T, int LX, int TY, int S, int NC = 4, int RP = 1, int XP = 0, int MODE = MODE_TEND, int RAG = 0>
 constexpr int tma_min_blocks() {
     using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
-    constexpr int by_smem = (int)((227u * 1024u) / L::SMEM);
+    constexpr int by_smem = (int)((227u * 1024u) / (L::SMEM + 1024u));   // 1 KB per CTA is the system's
     constexpr int by_threads = 2048 / L::THREADS;
-    constexpr int by_regs = (L::PD_SMEM && NC == 8)
-                                ? 65536 / (L::THREADS * PW_TMA_REGS_XP)
-                                : (NC * RP == 8 ? 65536 / (L::THREADS * PW_TMA_REGS8) : PW_TMA_MAX_MINB);
+    constexpr int by_regs =
+        (L::PD_SMEM && NC == 8)
+            ? 65536 / (L::THREADS * PW_TMA_REGS_XP)
+            : (NC * RP == 8 ? 65536 / (L::THREADS * PW_TMA_REGS8)
+                            : (MODE == MODE_STEP && !L::PACKED && !RAG ? 65536 / (L::THREADS * PW_STEP_REGS)
+                                                                       : PW_TMA_MAX_MINB));
     constexpr int m0 = by_smem < by_threads ? by_smem : by_threads;
     constexpr int m = m0 < by_regs ? m0 : by_regs;
     return m < 1 ? 1 : m;
@@ -840,16 +921,17 @@ struct MarchSmem {
         cnt = reinterpret_cast<uint32_t*>(bars + S) + 4;
         ctab = reinterpret_cast<float4*>(raw + L::ctab_off(sb));
     }
-    // one thread, then a CTA barrier
-    __device__ __forceinline__ void init(int tid) {
-        if (tid == 0) {
-            for (int s = 0; s < S; ++s) {
-                mbar_init(&bars[s], 1);
-                cnt[s] = 0;
-            }
-            flag[0] = 0;
-            fence_mbar_init();
+    // one thread; the others may touch the barriers after a CTA barrier
+    __device__ __forceinline__ void init_one() const {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&bars[s], 1);
+            cnt[s] = 0;
         }
+        flag[0] = 0;
+        fence_mbar_init();
+    }
+    __device__ __forceinline__ void init(int tid) const {
+        if (tid == 0) init_one();
         __syncthreads();
     }
 };
@@ -929,7 +1011,8 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
                                            const CUtensorMap* tm_v, const CUtensorMap* tm_w, T* __restrict__ o0,
                                            T* __restrict__ o1, T* __restrict__ o2, const GridDev& g, const int ox,
                                            const FoldedCoef& kc, const float dt, const int bx, const int by,
-                                           const int kb, const int ke, uint32_t& ring, int* __restrict__ err) {
+                                           const int kb, const int ke, uint32_t& ring, int* __restrict__ err,
+                                           const bool fresh = false) {
     using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
     using V = typename std::conditional<L::PACKED, float2, float>::type;
     constexpr int NV = XP ? NC / 2 : NC;   // values of type V per row vector
@@ -966,8 +1049,11 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
     auto slot = [&](int p) { return (int)((base + (uint32_t)p) % S); };
     auto parity = [&](int p) { return (uint32_t)(((base + (uint32_t)p) / S) & 1u); };
 
+    // (fresh: the CTA's first tile; the issuing thread initialises the ring
+    // itself, so the first planes are under way before the CTA's first barrier)
     int issued = 0;
     if (tid == 0) {
+        if (fresh) sm.init_one();
         prefetch_tensormap(tm_u);
         prefetch_tensormap(tm_v);
         prefetch_tensormap(tm_w);
@@ -978,10 +1064,17 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
     // previous tile of a persistent CTA is done with the table: every thread
     // has passed its last level's barrier)
     int tbase = pb;
-    if constexpr (L::CTAB) {
-        zcoef_fill(sm.ctab, kc, nz + 2, pb, min(ke, pb + L::CTAB_LEVELS - 1), tid, L::THREADS);
-        __syncthreads();
-    }
+    auto ctab_fill = [&](int lo) {
+        // (by every warp but the first, which issues the planes, where there are others)
+        constexpr int skip = L::WARPS > 1 ? 32 : 0;
+        if (tid < skip) return;
+        if constexpr (L::PACKED)
+            zcoef_fill(sm.ctab, kc, nz + 2, lo, min(ke, lo + L::CTAB_LEVELS - 1), tid - skip, L::THREADS - skip);
+        else
+            zcoef_fill1(sm.ctab, kc, nz + 2, lo, min(ke, lo + L::CTAB_LEVELS - 1), tid - skip, L::THREADS - skip);
+    };
+    ctab_fill(pb);
+    __syncthreads();
 
     const int r = row + 1;
     const int c0 = NC * xl + PADX;
@@ -1063,13 +1156,11 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
         constexpr bool FAST = decltype(fast)::value;
         constexpr bool SYNC = decltype(sync)::value;   // end the level with the CTA barrier
         lp = kk - pb;
-        if constexpr (L::CTAB) {
-            if (lp > 0 && lp % L::CTAB_LEVELS == 0) {
-                __syncthreads();   // every warp is done with the table's last level
-                tbase = kk;
-                zcoef_fill(sm.ctab, kc, nzp2, kk, min(ke, kk + L::CTAB_LEVELS - 1), tid, L::THREADS);
-                __syncthreads();
-            }
+        if (lp > 0 && lp % L::CTAB_LEVELS == 0) {
+            __syncthreads();   // every warp is done with the table's last level
+            tbase = kk;
+            ctab_fill(kk);
+            __syncthreads();
         }
         bool ok = true;
         if (!FAST && lp == 0) ok = mbar_wait_bounded(&bars[slot(0)], parity(0), kWaitLimitNs);
@@ -1115,20 +1206,23 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
                             return;
                         }
                     }
-                    Epilogue<T, MODE>::template store_field<NC>(of, o, a, g, j + half, i0, err);
+                    Epilogue<T, MODE>::template store_field<NC, (XP != 0)>(of, o, a, g, j + half, i0, err);
                 };
                 if (valid) field_row(0);
                 if (RP == 2 && valid2) field_row(1);
             };
-            // the same for the two-step kernel's three-field interface
-            auto out = [&](const V (&ru)[NV], const V (&rv)[NV], const V (&rw)[NV], const V (&u0)[NV],
-                           const V (&v0)[NV], const V (&w0)[NV]) {
-                outf(F_U, ru, u0);
-                outf(F_V, rv, v0);
-                outf(F_W, rw, w0);
-            };
             const bool first = !FAST && lp == 0, compute = FAST || ((kk >= kb) && (kk >= 2));
-            if constexpr (L::CTAB) {
+            if constexpr (!L::PACKED) {
+                const ZCoefTab1 zc{sm.ctab, tbase};
+                auto sideld = [&](int f, int up, int dr, int side) -> float {
+                    const T* P = rowp(f, up, dr);
+                    return ld1(side ? P + NC : P - 1);
+                };
+                using Nbr = typename std::conditional<MODE == MODE_TEND, NbrShflEdge<NV, LX, V, decltype(sideld)>,
+                                                      NbrLd<NV, V, decltype(sideld)>>::type;
+                const Nbr nbr{sideld, xl};
+                march_level_core<NV, V>(st, rowld, nbr, zc, outf, first, have_up, compute, kc, kk);
+            } else {
                 const ZCoefTab zc{sm.ctab, tbase};
                 if constexpr (XP && L::PD_SMEM) {
                     // thread tid's pairs 2m, 2m+1 of field f at float4 (f*NV/2 + m)*THREADS + tid
@@ -1154,8 +1248,6 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
                     const NbrShfl<NV, LX, V, decltype(edgeld)> nbr{edgeld, xl};
                     march_level_core<NV, V>(st, rowld, nbr, zc, outf, first, have_up, compute, kc, kk);
                 }
-            } else {
-                march_level<NV, LX>(st, rowld, edgeld, out, xl, first, have_up, compute, kc, kk, nzp2);
             }
         }
 #if PW_MARCH_SPLIT_ARRIVE
@@ -1254,7 +1346,7 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
 // One grid, one tile per CTA: blockIdx = (tile column, tile row, k segment).
 template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP, int RAG>
 __global__ void __launch_bounds__(TmaLayout<T, LX, TY, S, NC, RP, XP>::THREADS,
-                                  (tma_min_blocks<T, LX, TY, S, NC, RP, XP>()))
+                                  (tma_min_blocks<T, LX, TY, S, NC, RP, XP, MODE, RAG>()))
     tma_kernel(const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_v,
                const __grid_constant__ CUtensorMap tm_w, T* __restrict__ o0, T* __restrict__ o1,
                T* __restrict__ o2, const GridDev g, const int ox, const int nseg, const int seg0, const FoldedCoef kc,
@@ -1265,10 +1357,9 @@ __global__ void __launch_bounds__(TmaLayout<T, LX, TY, S, NC, RP, XP>::THREADS,
     const int kb = 1 + (int)(((long long)bz * g.nz) / nseg);
     const int ke = (int)(((long long)(bz + 1) * g.nz) / nseg);
     if (ke < kb) return;   // empty k segment (the host never launches one)
-    sm.init(threadIdx.y * 32 + threadIdx.x);
     uint32_t ring = 0;
     march_tile<T, LX, TY, S, MODE, NC, RP, XP, RAG>(sm, &tm_u, &tm_v, &tm_w, o0, o1, o2, g, ox, kc, dt, blockIdx.x,
-                                               blockIdx.y, kb, ke, ring, err);
+                                               blockIdx.y, kb, ke, ring, err, true);
 }
 
 // Instantiated single-grid launch shapes: (lanes per row, rows, stages, cells
@@ -1331,6 +1422,47 @@ static cudaError_t launch_tma_mode(const GridDev& g, int ox, const CUtensorMap* 
     PW_TMA_CONFIGS(PW_DISPATCH)
 #undef PW_DISPATCH
     return cudaErrorInvalidConfiguration;
+}
+
+template <typename T, int MODE, int RAG, int LX, int TY, int S, int NC, int RP, int XP>
+static int blocks_inst() {
+    int n = 0;
+    if constexpr (nc_ok<T, NC, RP, XP>()) {
+        auto kern = tma_kernel<T, LX, TY, S, MODE, NC, RP, XP, RAG>;
+        using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
+        if (set_smem_attr_once(kern, (int)L::SMEM) != cudaSuccess) return 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, L::THREADS, L::SMEM) != cudaSuccess) return 0;
+    }
+    return n;
+}
+
+// CTAs of the k-march resident per SM for a launch shape (0: no such kernel).
+template <typename T, int MODE>
+static int blocks_per_sm_mode(const TmaConfig& c) {
+#define PW_OCC(LX_, TY_, S_, NC_, RP_, XP_)                                                            \
+    if (c.lx == LX_ && c.ty == TY_ && c.stages == S_ && c.nc == NC_ && c.rp == RP_ && c.xp == XP_)     \
+        return blocks_inst<T, MODE, PW_OCC_RAG, LX_, TY_, S_, NC_, RP_, XP_>();
+    if (c.rag) {
+#define PW_OCC_RAG 1
+        PW_TMA_RAGGED(PW_OCC)
+#undef PW_OCC_RAG
+        return 0;
+    }
+#define PW_OCC_RAG 0
+    PW_TMA_CONFIGS(PW_OCC)
+#undef PW_OCC_RAG
+#undef PW_OCC
+    return 0;
+}
+
+template <int MODE>
+static int blocks_per_sm_dtype(pw_dtype_t dt, const TmaConfig& c) {
+    switch (dt) {
+        case PW_F32: return blocks_per_sm_mode<float, MODE>(c);
+        case PW_BF16: return blocks_per_sm_mode<__nv_bfloat16, MODE>(c);
+        case PW_F16: return blocks_per_sm_mode<__half, MODE>(c);
+    }
+    return 0;
 }
 
 }  // namespace pw

@@ -37,4 +37,6 @@ cudaError_t launch_step_tma(pw_dtype_t dt, const GridDev& g, int ox, const CUten
     return cudaErrorInvalidValue;
 }
 
+int step_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c) { return blocks_per_sm_dtype<MODE_STEP>(dt, c); }
+
 }  // namespace pw

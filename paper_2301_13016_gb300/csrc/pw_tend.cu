@@ -61,32 +61,7 @@ size_t tma_smem_bytes(pw_dtype_t dt, const TmaConfig& c) {
     return 0;
 }
 
-template <typename T>
-static int blocks_per_sm_t(const TmaConfig& c) {
-    int n = 0;
-#define PW_OCC(LX_, TY_, S_, NC_, RP_, XP_)                                                           \
-    if constexpr (nc_ok<T, NC_, RP_, XP_>())                                                           \
-        if (c.lx == LX_ && c.ty == TY_ && c.stages == S_ && c.nc == NC_ && c.rp == RP_ && c.xp == XP_) { \
-            auto kern = tma_kernel<T, LX_, TY_, S_, MODE_TEND, NC_, RP_, XP_, 0>;                         \
-            using L = TmaLayout<T, LX_, TY_, S_, NC_, RP_, XP_>;                                       \
-            if (set_smem_attr_once(kern, (int)L::SMEM) != cudaSuccess) return 0;                       \
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, L::THREADS, L::SMEM) != cudaSuccess) \
-                return 0;                                                                              \
-            return n;                                                                                  \
-        }
-    PW_TMA_CONFIGS(PW_OCC)
-#undef PW_OCC
-    return 0;
-}
-
-int tma_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c) {
-    switch (dt) {
-        case PW_F32: return blocks_per_sm_t<float>(c);
-        case PW_BF16: return blocks_per_sm_t<__nv_bfloat16>(c);
-        case PW_F16: return blocks_per_sm_t<__half>(c);
-    }
-    return 0;
-}
+int tma_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c) { return blocks_per_sm_dtype<MODE_TEND>(dt, c); }
 
 int tma_box_width(pw_dtype_t dt, int lx, int nc) { return nc * lx + 2 * (16 / (int)dtype_size(dt)); }
 
