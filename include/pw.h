@@ -149,9 +149,12 @@ pw_status_t pw_set_kernel(pw_handle_t h, int32_t kind);
  * (lanes_x, ty, stages, cells, rows_per_thread) = (32, 4, 4, 4, 1); all zero
  * restores the automatic choice, which depends on the call: (32, 4, 4, 4, 1)
  * for FP32; (16, 8, 4, 8, 3) for 16-bit storage (fused steps: when nx is a
- * multiple of 8, else (32, 4, 4, 4, 3)); (16, 4, 4, 4, 1) when nx <= 64; nseg
- * the count that best fills the last wave of CTAs per plane marched
- * (segments of >= 2 levels; more segments only for a >= 3 % gain).
+ * multiple of 8, else (32, 4, 4, 4, 3)); (16, 4, 4, 4, 1) when nx <= 64; from
+ * 2^18 cells up narrower tiles of as many cells, (16, 8, 4, 4, 1) and
+ * (8, 16, 4, 4, 1) for FP32, (8, 16, 4, 8, 3), resp. (16, 8, 4, 4, 3), for 16
+ * bits, where they are estimated to be faster (fewer cells beyond nx); nseg the
+ * count estimated to fill the GPU best (segments of >= 2 levels; narrower tiles
+ * and more segments only for a gain of 1.5 %).
  * Instantiated (lanes_x, ty, stages, cells, rows_per_thread): (32,4,4,4,1)
  * (32,8,3,4,1) (32,8,4,4,1) (32,8,6,4,1) (32,16,3,4,1) (16,4,4,4,1)
  * (16,8,4,4,1), and for 16-bit storage also (16,4,4,8,1) (16,8,4,8,1)

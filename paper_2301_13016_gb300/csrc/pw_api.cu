@@ -245,85 +245,91 @@ static pw_status_t check_device_ptrs(pw_handle_t h, const void* const* ps, int n
 // Launch shape of the TMA kernel for the source terms (step = false) or the
 // fused step (step = true).  A shape the user fixed (pw_set_tma_config) is used
 // as given, unset fields at the scalar defaults (32 lanes x 4 cells x 4 rows, 4
-// stages, one row per thread).  Otherwise the shape measured fastest on GB300
-// (2048^2 x 64):
-//   FP32:                       32 lanes x 4 cells x 4 rows (HBM-bound);
+// stages, one row per thread).  Otherwise 4 stages and one of these (lanes x
+// cells x rows), with the k segments, whichever march_cost puts lowest:
+//   nx <= 64:                   16 x 4 x 4 alone;
+//   FP32:                       32 x 4 x 4, 16 x 4 x 8, 8 x 4 x 16;
 //   16-bit (source terms; steps when nx % 8 = 0):
-//                               16 lanes x 8 cells x 8 rows, each thread's
-//                               cells packed as FP32x2 pairs along x (BF16
-//                               401, FP16 400 Gcell/s; two rows per thread
-//                               315, 331);
-//   16-bit steps, nx % 8 = 4:   32 lanes x 4 cells x 4 rows in x pairs;
-//   nx <= 64:                   16 lanes x 4 cells x 4 rows;
-// 4 stages, and the k segments chosen below.
+//                               16 x 8 x 8, 8 x 8 x 16, a thread's cells
+//                               packed as FP32x2 pairs along x;
+//   16-bit steps otherwise:     32 x 4 x 4, 16 x 4 x 8 in x pairs (the 8-cell
+//                               form spills with ragged rows: 335 us a step
+//                               against 218 at 1021 x 1023 x 61).
+// The first of each line is the fastest on whole tiles; the narrower ones cover
+// fewer cells beyond nx.  FP32 source terms, first shape alone against the
+// choice: 160x824x41 39.2 -> 29.1 us, 184x1280x21 33.6 -> 27.6, 776x184x29 25.4
+// -> 21.3, 320x1120x26 48.0 -> 45.5; BF16 320x1216x69 94.9 -> 82.8, 1056x1552x24
+// 122 -> 115, 512x512x64 (segments alone) 61 -> 55.  Grids below kShapeMinCells
+// keep the first shape: a call of that size is launch and latency.
+constexpr long long kShapeMinCells = 1 << 18;
+
+// Estimated time of a march in units of one level of a full SM: `slots` CTAs
+// fit the GPU, each marches its levels after a start that costs as much as 1.6
+// of them (x pairs, whose levels take longer: 0.8); a last wave that leaves SMs
+// with r of their R slots takes 0.7 + 0.3 r / R of a full one (x pairs: 0.45 +
+// 0.55 r / R), as fewer CTAs on an SM each run faster.  Fitted to a sweep of
+// shapes and segments over 31 grids (64^3 to 1056 x 1552 x 24): in the mean the
+// choice is within 1 % (FP32 source terms), 2 % (16-bit), 3 to 4 % (steps) of
+// the sweep's best, where counting whole waves of (levels + 2) was 8 % off.
+static double march_cost(const pw_grid_t& gr, const TmaConfig& c, int n, int sms, int bps) {
+    const long long tiles = (long long)((gr.nx + c.nc * c.lx - 1) / (c.nc * c.lx)) * ((gr.ny + c.ty - 1) / c.ty);
+    const long long ctas = tiles * n, slots = (long long)sms * bps;
+    const long long full = ctas / slots, rem = ctas - full * slots;
+    const double w = c.xp ? 0.45 : 0.7;
+    const double last = rem ? w + (1.0 - w) * (double)((rem + sms - 1) / sms) / bps : 0.0;
+    return ((gr.nz + n - 1) / n + (c.xp ? 0.8 : 1.6)) * ((double)full + last) * bps * (c.nc * c.lx) * c.ty;
+}
+
 static TmaConfig choose_tma(pw_handle_t h, bool step) {
     TmaConfig& cache = h->tma_auto[step ? 1 : 0];
     if (cache.ty) return cache;
     const TmaConfig& u = h->tma_user;
     const pw_grid_t& gr = h->grid;
-    TmaConfig c;
-    if (u.lx || u.nc || u.ty || u.stages || u.rp) {
-        c.lx = u.lx ? u.lx : 32;
-        c.nc = u.nc ? u.nc : 4;
-        c.ty = u.ty ? u.ty : 4;
-        c.stages = u.stages ? u.stages : 4;
-        c.rp = u.rp ? u.rp : 1;
-        if (c.rp == 3) {   // one row per thread, cells paired along x
-            c.rp = 1;
-            c.xp = 1;
-        }
+    TmaConfig cand[3];
+    int nc = 0;
+    auto add = [&](int lx, int cells, int ty, int xp, int rp) {
+        TmaConfig c{lx, ty, 4, 1, cells};
+        c.rp = rp;
+        c.xp = xp;
+        cand[nc++] = c;
+    };
+    if (u.lx || u.nc || u.ty || u.stages || u.rp) {   // rows_per_thread 3: one row, cells paired along x
+        add(u.lx ? u.lx : 32, u.nc ? u.nc : 4, u.ty ? u.ty : 4, u.rp == 3, (u.rp && u.rp != 3) ? u.rp : 1);
+        if (u.stages) cand[0].stages = u.stages;
     } else {
-        const bool half = dtype_size(gr.dtype) == 2;
-        c.rag = gr.nx % 4 != 0;
-        c.lx = 32;
-        c.nc = 4;
-        c.ty = 4;
-        c.stages = 4;
-        c.rp = 1;
+        const bool half = dtype_size(gr.dtype) == 2, more = (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells;
         if (gr.nx <= 64) {
-            c.lx = 16;
-        } else if (half && (!step || gr.nx % 8 == 0 || c.rag)) {
-            c.lx = 16;   // x pairs of 8 cells: tiles of 128 columns
-            c.nc = 8;
-            c.ty = 8;
-            c.xp = 1;
-        } else if (half) {
-            c.xp = 1;    // x pairs of 4 cells
+            add(16, 4, 4, 0, 1);
+        } else if (!half) {
+            add(32, 4, 4, 0, 1);
+            if (more) add(16, 4, 8, 0, 1);
+            if (more) add(8, 4, 16, 0, 1);
+        } else if (!step || gr.nx % 8 == 0) {
+            add(16, 8, 8, 1, 1);
+            if (more) add(8, 8, 16, 1, 1);
+        } else {
+            add(32, 4, 4, 1, 1);
+            if (more) add(16, 4, 8, 1, 1);
         }
+        for (int q = 0; q < nc; ++q) cand[q].rag = gr.nx % 4 != 0;
     }
-    if (u.nseg) {
-        c.nseg = u.nseg;
-    } else {
-        const long long tiles =
-            (long long)((gr.nx + c.nc * c.lx - 1) / (c.nc * c.lx)) * ((gr.ny + c.ty - 1) / c.ty);
+    TmaConfig best = cand[0];
+    double lowest = 0.0;
+    for (int q = 0; q < nc; ++q) {
+        TmaConfig c = cand[q];
         int bps = step ? step_blocks_per_sm(gr.dtype, c) : tma_blocks_per_sm(gr.dtype, c);
         if (bps < 1) bps = 1;
-        const long long slots = (long long)h->num_sms * bps;
-        // the count that minimises (waves of CTAs) x (planes each CTA marches:
-        // its levels plus the two beyond them), down to 2 levels per segment;
-        // more segments only for a gain of >= 3 %; and a single wave is
-        // widened to two when that costs <= 5 % (one partial wave leaves SMs
-        // with unequal CTA counts).  Measured on GB300 (FP32, 64 levels,
-        // Gcell/s): 256^2 145 -> 181 (4 segments instead of 16), 1024^2
-        // 236 -> 249 (2 instead of 1), 512^2 216 (1 segment) / 221 (2); 64^3
-        // keeps 32 segments of 2 levels (4.0 us per call in a CUDA graph, 7.0
-        // with 8)
-        auto waves = [&](int n) { return (tiles * n + slots - 1) / slots; };
-        auto cost = [&](int n) { return (double)waves(n) * ((double)gr.nz / n + 2.0); };
-        int nseg = 1;
-        for (int n = 2; gr.nz / n >= 2; ++n)
-            if (cost(n) < 0.97 * cost(nseg)) nseg = n;
-        if (waves(nseg) < 2)
-            for (int n = nseg + 1; gr.nz / n >= 2; ++n)
-                if (waves(n) >= 2) {
-                    if (cost(n) <= 1.05 * cost(nseg)) nseg = n;
-                    break;
-                }
-        c.nseg = nseg;
+        const int lo = u.nseg ? u.nseg : 1, hi = u.nseg ? u.nseg : std::max(1, gr.nz / 2);
+        for (c.nseg = lo; c.nseg <= hi; ++c.nseg) {
+            const double cost = march_cost(gr, c, c.nseg, h->num_sms, bps);
+            if (lowest > 0.0 && !(cost < 0.985 * lowest)) continue;   // narrower or more segments only for a gain
+            lowest = cost;
+            best = c;
+        }
     }
-    if (c.nseg > gr.nz / 2) c.nseg = std::max(1, gr.nz / 2);
-    cache = c;
-    return c;
+    if (best.nseg > gr.nz / 2) best.nseg = std::max(1, gr.nz / 2);
+    cache = best;
+    return best;
 }
 
 // TMA k-march or generic kernel for the source terms and the steps: what

@@ -1377,7 +1377,14 @@ __global__ void __launch_bounds__(TmaLayout<T, LX, TY, S, NC, RP, XP>::THREADS,
 
 // Shapes for a width that is no multiple of 4 (RAG kernels): the automatic
 // ones only; a shape the caller fixed keeps to the generic kernel there.
-#define PW_TMA_RAGGED(X) X(32, 4, 4, 4, 1, 0) X(16, 4, 4, 4, 1, 0) X(16, 8, 4, 8, 1, 1)
+#define PW_TMA_RAGGED(X) X(32, 4, 4, 4, 1, 0) X(16, 8, 4, 4, 1, 0) X(8, 16, 4, 4, 1, 0) X(16, 4, 4, 4, 1, 0)   \
+    X(16, 8, 4, 8, 1, 1) X(8, 16, 4, 8, 1, 1) X(32, 4, 4, 4, 1, 1) X(16, 8, 4, 4, 1, 1)
+// ... of which 16-bit storage takes the narrow scalar one, 8-cell x pairs for
+// the source terms and 4-cell ones for steps.
+template <typename T, int MODE, int LX, int TY, int NC, int XP>
+constexpr bool rag_ok() {
+    return sizeof(T) == 4 ? XP == 0 : (XP ? NC == (MODE == MODE_TEND ? 8 : 4) : LX * TY == 64);
+}
 
 template <typename T, int NC, int RP, int XP = 0>
 constexpr bool nc_ok() { return (NC == 4 && RP == 1 && XP == 0) || sizeof(T) == 2; }
@@ -1386,7 +1393,7 @@ template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP, i
 static cudaError_t launch_tma_inst(const GridDev& g, int ox, const CUtensorMap* maps, void* o0, void* o1,
                                    void* o2, const Scales& sc, const CoefDev& cf, float dt, int* err, int nseg,
                                    int seg0, int seg_count, cudaStream_t s) {
-  if constexpr (!nc_ok<T, NC, RP, XP>()) {
+  if constexpr (!nc_ok<T, NC, RP, XP>() || (RAG && !rag_ok<T, MODE, LX, TY, NC, XP>())) {
     return cudaErrorInvalidConfiguration;
   } else {
     using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
@@ -1427,7 +1434,7 @@ static cudaError_t launch_tma_mode(const GridDev& g, int ox, const CUtensorMap* 
 template <typename T, int MODE, int RAG, int LX, int TY, int S, int NC, int RP, int XP>
 static int blocks_inst() {
     int n = 0;
-    if constexpr (nc_ok<T, NC, RP, XP>()) {
+    if constexpr (nc_ok<T, NC, RP, XP>() && (!RAG || rag_ok<T, MODE, LX, TY, NC, XP>())) {
         auto kern = tma_kernel<T, LX, TY, S, MODE, NC, RP, XP, RAG>;
         using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
         if (set_smem_attr_once(kern, (int)L::SMEM) != cudaSuccess) return 0;

@@ -77,6 +77,34 @@ def test_ragged_steps_match_oracle(nx, halo, dtype, tol):
             assert torch.equal(v[:, :, halo + nx + d - 1], v[:, :, halo + d - 1])
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("shape", [(160, 824, 41), (184, 1280, 21), (320, 512, 21), (1056, 300, 24), (164, 824, 41)])
+def test_automatic_shapes_give_the_first_shapes_bits(shape, dtype):
+    """Grids large enough for the choice among tile widths: source terms and a
+    step equal, bit for bit, those of the first shape in one k segment."""
+    nx, ny, nz = shape
+    c = inputs.make_coeffs(nz, anelastic=True)
+    g = pwlib.Grid(nx, ny, nz, dtype=dtype)
+    f = inputs.random_fields(nx, ny, nz)
+    dev = [g.from_dense(x) for x in f]
+    out = []
+    for fixed in (False, True):
+        h = pwlib.PW(g, c)
+        for call in (0, 1):
+            if fixed:
+                cells = 4 if dtype == "f32" or (call and nx % 8) else 8
+                h.set_tma_config(ty=4 if cells == 4 else 8, stages=4, nseg=1, lanes_x=32 if cells == 4 else 16,
+                                 cells=cells, rows=1 if dtype == "f32" else 3)
+            res = [g.alloc(fill=NAN) for _ in range(3)]
+            h.step_to(*dev, *res, 0.25) if call else h.tendencies(*dev, *res)
+            h.sync()
+            assert h.last_kernel == 2
+            out.append([g.view(t)[1:-1].cpu() for t in res])
+    for a, b in zip(out[0] + out[1], out[2] + out[3]):
+        assert torch.equal(a.view(torch.int16 if dtype == "bf16" else torch.int32),
+                           b.view(torch.int16 if dtype == "bf16" else torch.int32))
+
+
 def test_ragged_refusals_unchanged():
     """pw_set_kernel(2), two steps per pass and a fixed launch shape still treat
     such a width as not eligible for the k-march."""
