@@ -57,8 +57,12 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
+// Which cells of a field a tensor map covers: the whole padded field (the
+// k-march), or one of the adjoint's (adj_map).
+enum { MAP_FIELD = 0, MAP_ADJ = 1 };
 struct MapCacheEntry {
     const void* ptr = nullptr;
+    int kind = MAP_FIELD;
     int box_w = 0, box_h = 0;
     CUtensorMap map;
 };
@@ -84,7 +88,7 @@ struct pw_handle_s {
     Step2Config step2_user{0, 0, 0, 0};
     Step2Config step2_auto{0, 0, 0, 0};   // ty == 0: not chosen yet
     AdjConfig adj_user{0, 0, 0, 0};       // TMA adjoint shape; 0 = automatic
-    AdjConfig adj_auto{0, 0, 0, 0};       // the shape in use; na == 0: not chosen yet
+    AdjConfig adj_auto[2] = {};           // the shape in use (periodic, open mode); na == 0: not chosen yet
     MapCacheEntry maps[8];
     int map_next = 0;   // round-robin replacement
     // field pointers already found to be device memory of this handle's GPU
@@ -173,7 +177,7 @@ bool pw::is_device_ptr(const void* p, int device) {
 // handle's cache of recently encoded maps.
 static pw_status_t encode_map_box(pw_handle_t h, const void* ptr, int box_w, int box_h, CUtensorMap* out) {
     for (auto& c : h->maps)
-        if (c.ptr == ptr && c.box_w == box_w && c.box_h == box_h) {
+        if (c.ptr == ptr && c.kind == MAP_FIELD && c.box_w == box_w && c.box_h == box_h) {
             *out = c.map;
             return PW_OK;
         }
@@ -182,6 +186,7 @@ static pw_status_t encode_map_box(pw_handle_t h, const void* ptr, int box_w, int
     pw_status_t st = encode_tensor_map_box(h->grid, ptr, box_w, box_h, out);
     if (st != PW_OK) return st;
     e.ptr = ptr;
+    e.kind = MAP_FIELD;
     e.box_w = box_w;
     e.box_h = box_h;
     e.map = *out;
@@ -203,26 +208,69 @@ pw_status_t pw::encode_tensor_map(const pw_grid_t& g, const void* ptr, int lx, i
 // box_w x box_h x 1; out-of-range elements read as zero.
 pw_status_t pw::encode_tensor_map_box(const pw_grid_t& g, const void* ptr, int box_w, int box_h, CUtensorMap* out,
                                       int l2_promotion) {
-    auto fn = encode_fn();
-    if (!fn) return fail(PW_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    if (inject_failure(INJECT_TENSOR_MAP)) return fail(PW_ERR_CUDA, "cuTensorMapEncodeTiled failed (injected)");
     int ox = 0;
     const char* why = "";
     // (the callers decide about widths: a box may run past the row's end)
     if (!tma_layout_ok(g, &ox, &why, true)) return fail(PW_ERR_UNSUPPORTED, "layout not TMA-eligible: %s", why);
+    return encode_tensor_map_dims(g, ptr, {ox + g.nx + g.halo + 1, g.ny + 2 * g.halo, g.nz + 2}, box_w, box_h, out,
+                                  l2_promotion);
+}
+
+pw_status_t pw::encode_tensor_map_dims(const pw_grid_t& g, const void* base, const long long (&n)[3], int box_w,
+                                       int box_h, CUtensorMap* out, int l2_promotion) {
+    auto fn = encode_fn();
+    if (!fn) return fail(PW_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    if (inject_failure(INJECT_TENSOR_MAP)) return fail(PW_ERR_CUDA, "cuTensorMapEncodeTiled failed (injected)");
     const size_t es = dtype_size(g.dtype);
     CUtensorMapDataType dt = g.dtype == PW_F32    ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                              : g.dtype == PW_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                                   : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-    cuuint64_t dims[3] = {(cuuint64_t)(ox + g.nx + g.halo + 1), (cuuint64_t)(g.ny + 2 * g.halo),
-                          (cuuint64_t)(g.nz + 2)};
+    cuuint64_t dims[3] = {(cuuint64_t)n[0], (cuuint64_t)n[1], (cuuint64_t)n[2]};
     cuuint64_t strides[2] = {(cuuint64_t)(g.pitch_j * es), (cuuint64_t)(g.pitch_k * es)};
     cuuint32_t box[3] = {(cuuint32_t)box_w, (cuuint32_t)box_h, 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = fn(out, dt, 3, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    CUresult r = fn(out, dt, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                     CU_TENSOR_MAP_SWIZZLE_NONE, (CUtensorMapL2promotion)l2_promotion,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(PW_ERR_CUDA, "cuTensorMapEncodeTiled failed (CUresult %d)", (int)r);
+    return PW_OK;
+}
+
+// A tensor map of the TMA adjoint for field f of (u, v, w, lsu, lsv, lsw), and
+// where levels, rows and columns lie in such maps (AdjGeom).  Periodic mode:
+// whole rows with their halos, levels 1..nz of u, v, w, 2..nz of lsu and lsv,
+// 2..nz-1 of lsw.  Open mode: u, v, w on columns -3..nx+1 (-3 is the first
+// 16-byte boundary at or before column 0; interior rows start on one) and rows
+// 0..ny+1, the sensitivities on the interior.
+static AdjGeom adj_geom(const pw_grid_t& g, int ox, bool open) {
+    if (open) return AdjGeom{3, 0, -1, -1, -1, -2};
+    return AdjGeom{ox, g.halo - 1, -1, ox, g.halo - 1, -2};
+}
+static pw_status_t adj_map(pw_handle_t h, int f, const void* ptr, bool open, int ox, int box_w, int box_h,
+                           CUtensorMap* out) {
+    const int kind = MAP_ADJ + 2 * (f < 3 ? 0 : (f < 5 ? 1 : 2)) + (open ? 1 : 0);
+    for (auto& c : h->maps)
+        if (c.ptr == ptr && c.kind == kind && c.box_w == box_w && c.box_h == box_h) {
+            *out = c.map;
+            return PW_OK;
+        }
+    const pw_grid_t& g = h->grid;
+    const AdjGeom ge = adj_geom(g, ox, open);
+    // the map's first element: level, row and column with coordinate 0
+    const long long k = f < 3 ? -ge.fz : -ge.lz, j = f < 3 ? -ge.fy : -ge.ly, i = f < 3 ? -ge.fx : -ge.lx;
+    const float* base = static_cast<const float*>(ptr) + g.origin + k * g.pitch_k + j * g.pitch_j + i;
+    const long long levels = f < 3 ? g.nz : (f < 5 ? g.nz - 1 : g.nz - 2);
+    const long long rows = !open ? g.ny + 2LL * g.halo : (f < 3 ? g.ny + 2 : g.ny);
+    const long long cols = !open ? ox + g.nx + g.halo + 1LL : (f < 3 ? g.nx + 5 : g.nx);
+    pw_status_t st = encode_tensor_map_dims(g, base, {cols, rows, levels}, box_w, box_h, out);
+    if (st != PW_OK) return st;
+    MapCacheEntry& e = h->maps[h->map_next];
+    h->map_next = (h->map_next + 1) % (int)(sizeof(h->maps) / sizeof(h->maps[0]));
+    e.ptr = ptr;
+    e.kind = kind;
+    e.box_w = box_w;
+    e.box_h = box_h;
+    e.map = *out;
     return PW_OK;
 }
 
@@ -584,39 +632,47 @@ static Step2Config choose_step2(pw_handle_t h) {
     return c;
 }
 
-// Launch shape of the TMA adjoint: each field the user fixed, else the
-// automatic shape's.  k segments (automatic): the count that minimises the
-// waves of CTAs times the planes each CTA marches (its levels plus the two
-// it reads beyond them); segments keep >= 8 levels.  The adjoint holds few
-// CTAs per SM (2 to 5), so a partly filled last wave costs much: at
-// 512^2 x 64 with 64 x 4 tiles, 1024 CTAs fill 760 slots 1.35 times, and two
-// segments turn that into 2.7 waves of half-length CTAs.
-static AdjConfig choose_adjoint(pw_handle_t h) {
-    if (h->adj_auto.na) return h->adj_auto;
+// Launch shape of the TMA adjoint (periodic or open mode): each field the user
+// fixed, else 4 cells x 6 rows with 4 slots for grids below kShapeMinCells, and
+// above 32 lanes x 8 rows or 16 lanes x 16 rows with 3 slots; k segments
+// (automatic) of >= 4 levels.  Shape and segments as for the k-march: the
+// lowest estimated time, a segment's start costing 2.5 levels (two planes
+// more than its levels, the priming level).
+static AdjConfig choose_adjoint(pw_handle_t h, bool open) {
+    AdjConfig& cache = h->adj_auto[open ? 1 : 0];
+    if (cache.na) return cache;
     const AdjConfig d = adjoint_default_config();
     const AdjConfig& u = h->adj_user;
-    AdjConfig c{u.na ? u.na : d.na, u.ty ? u.ty : d.ty, u.stages ? u.stages : d.stages, u.nseg};
     const pw_grid_t& gr = h->grid;
-    if (!c.nseg) {
-        const int tx = 32 * c.na;
-        const long long tiles = (long long)((gr.nx + tx - 1) / tx) * ((gr.ny + c.ty - 1) / c.ty);
-        int bps = adjoint_blocks_per_sm(c);
-        if (bps < 1) bps = 1;
+    AdjConfig cand[2] = {AdjConfig{u.na ? u.na : d.na, u.ty ? u.ty : d.ty, u.stages ? u.stages : d.stages, 0, 32}};
+    int nc = 1;
+    if (open || (!u.na && !u.ty && !u.stages && (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells)) {
+        cand[0] = AdjConfig{4, 8, 3, 0, 32};
+        cand[1] = AdjConfig{4, 16, 3, 0, 16};
+        nc = 2;
+    }
+    AdjConfig best = cand[0];
+    double lowest = 0.0;
+    const int wx = open ? gr.nx + 5 : gr.nx, wy = open ? gr.ny + 2 : gr.ny;
+    for (int q = 0; q < nc; ++q) {
+        AdjConfig c = cand[q];
+        const int tx = c.lx * c.na;
+        const long long tiles = (long long)((wx + tx - 1) / tx) * ((wy + c.ty - 1) / c.ty);
+        const int bps = std::max(1, adjoint_blocks_per_sm(c, open));
         const long long slots = (long long)h->num_sms * bps;
-        c.nseg = 1;
-        double best = 0.0;
-        for (int n = 1; n <= 16 && (n == 1 || gr.nz / n >= 8); ++n) {
-            const long long waves = (tiles * n + slots - 1) / slots;
-            const double cost = (double)waves * ((double)gr.nz / n + 2.0);
-            if (n == 1 || cost < 0.999 * best) {
-                best = cost;
-                c.nseg = n;
-            }
+        const int lo = u.nseg ? u.nseg : 1, hi = u.nseg ? u.nseg : std::max(1, gr.nz / 4);
+        for (c.nseg = lo; c.nseg <= hi; ++c.nseg) {
+            const long long full = tiles * c.nseg / slots, rem = tiles * c.nseg - full * slots;
+            const double last = rem ? 0.6 + 0.4 * (double)((rem + h->num_sms - 1) / h->num_sms) / bps : 0.0;
+            const double cost = ((gr.nz + c.nseg - 1) / c.nseg + 2.5) * ((double)full + last) * bps * tx * c.ty;
+            if (lowest > 0.0 && !(cost < 0.985 * lowest)) continue;
+            lowest = cost;
+            best = c;
         }
     }
-    if (c.nseg > gr.nz) c.nseg = gr.nz;
-    h->adj_auto = c;
-    return c;
+    if (best.nseg > gr.nz) best.nseg = gr.nz;
+    cache = best;
+    return best;
 }
 
 pw_status_t pw_set_adjoint_config(pw_handle_t h, int32_t cells, int32_t ty, int32_t stages, int32_t nseg) {
@@ -624,18 +680,18 @@ pw_status_t pw_set_adjoint_config(pw_handle_t h, int32_t cells, int32_t ty, int3
     if (cells < 0 || ty < 0 || stages < 0) return fail(PW_ERR_ARG, "cells, ty and stages must be >= 0");
     if (nseg < 0 || nseg > h->grid.nz) return fail(PW_ERR_ARG, "nseg must be in 0..nz");
     const AdjConfig d = adjoint_default_config();
-    const AdjConfig c{cells ? cells : d.na, ty ? ty : d.ty, stages ? stages : d.stages, nseg};
+    const AdjConfig c{cells ? cells : d.na, ty ? ty : d.ty, stages ? stages : d.stages, nseg, 32};
     if (!adjoint_config_supported(c))
         return fail(PW_ERR_UNSUPPORTED, "no TMA adjoint instance for cells=%d ty=%d stages=%d", c.na, c.ty,
                     c.stages);
     h->adj_user = AdjConfig{cells, ty, stages, nseg};
-    h->adj_auto = AdjConfig{0, 0, 0, 0};
+    h->adj_auto[0] = h->adj_auto[1] = AdjConfig{};
     return PW_OK;
 }
 
 pw_status_t pw_get_adjoint_config(pw_handle_t h, int32_t out[4]) {
     if (!h || !out) return fail(PW_ERR_ARG, "handle or out is NULL");
-    const AdjConfig c = choose_adjoint(h);
+    const AdjConfig c = choose_adjoint(h, false);
     out[0] = c.na;
     out[1] = c.ty;
     out[2] = c.stages;
@@ -902,8 +958,7 @@ static pw_status_t step_pass(pw_handle_t h, const GridDev& g, const void* const*
         }
         e = launch_step_tma(dtp, g, ox, maps, dst[0], dst[1], dst[2], sc, cf, dt, h->d_err, c, s);
         // the single-step k-march writes the images of a one-cell halo only
-        for (int q = 0; q < 3 && e == cudaSuccess && g.halo != 1; ++q)
-            e = launch_fill_halo(dtp, g, dst[q], h->num_sms, s);
+        if (e == cudaSuccess && g.halo != 1) e = launch_fill_halo(dtp, g, dst, 3, h->num_sms, s);
     } else {
         e = launch_step_generic(dtp, g, src[0], src[1], src[2], dst[0], dst[1], dst[2], sc, scaled, cf, dt,
                                 h->num_sms, s);
@@ -967,8 +1022,8 @@ pw_status_t pw_step(pw_handle_t h, void* u, void* v, void* w, void* tmp_u, void*
     CoefDev cf{h->tcx, h->tcy, h->d_tz};
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const pw_dtype_t dtp = h->grid.dtype;
-    for (int q = 0; q < 3; ++q) {
-        cudaError_t e = launch_fill_halo(dtp, g, bufs[q], h->num_sms, s);
+    {
+        cudaError_t e = launch_fill_halo(dtp, g, bufs, 3, h->num_sms, s);
         if (e != cudaSuccess) return cuda_fail(e, "halo fill launch");
     }
     int ox = 0;
@@ -1055,23 +1110,30 @@ pw_status_t pw_adjoint(pw_handle_t h, const void* u, const void* v, const void* 
     const char* why = "";
     bool ptrs_ok = true;
     for (auto p : ins) ptrs_ok = ptrs_ok && aligned16(p);
-    if ((flags & PW_ADJ_PERIODIC) && h->kernel_kind != 1 && ptrs_ok && tma_layout_ok(h->grid, &ox, &why)) {
-        // TMA k-march adjoint: the sensitivities need periodic halos too
+    const bool open = !(flags & PW_ADJ_PERIODIC);
+    const AdjConfig& au = h->adj_user;
+    for (auto p : outs) ptrs_ok = ptrs_ok && aligned16(p);
+    // the open mode takes any width, with the automatic shape
+    const bool shape_ok = !open || !(au.na || au.ty || au.stages || au.nseg);
+    if (h->kernel_kind != 1 && ptrs_ok && shape_ok && tma_layout_ok(h->grid, &ox, &why, open)) {
         const GridDev g = to_dev(h->grid);
-        for (int q = 3; q < 6; ++q) {
-            cudaError_t e = launch_fill_halo(PW_F32, g, const_cast<void*>(ins[q]), h->num_sms, s);
+        if (!open) {   // the sensitivities need periodic halos too
+            void* ls[3] = {const_cast<void*>(lsu), const_cast<void*>(lsv), const_cast<void*>(lsw)};
+            cudaError_t e = launch_fill_halo(PW_F32, g, ls, 3, h->num_sms, s);
             if (e != cudaSuccess) return cuda_fail(e, "sensitivity halo fill");
         }
         CUtensorMap maps[6];
-        const AdjConfig ac = choose_adjoint(h);
+        const AdjConfig ac = choose_adjoint(h, open);
         for (int q = 0; q < 6; ++q) {
-            pw_status_t st = encode_map(h, ins[q], 32, ac.ty, &maps[q], ac.na);
+            pw_status_t st = adj_map(h, q, ins[q], open, ox, ac.lx * ac.na + 8, ac.ty + 2, &maps[q]);
             if (st != PW_OK) return st;
         }
-        const int nseg = ac.nseg;
-        cudaError_t e = launch_adjoint_tma(g, ox, maps, (float*)gu, (float*)gv, (float*)gw, alpha,
+        const float* q6[6] = {(const float*)u,   (const float*)v,   (const float*)w,
+                              (const float*)lsu, (const float*)lsv, (const float*)lsw};
+        float* g3[3] = {(float*)gu, (float*)gv, (float*)gw};
+        cudaError_t e = launch_adjoint_tma(g, adj_geom(h->grid, ox, open), open, maps, q6, g3, alpha,
                                            (flags & PW_ADJ_ACCUMULATE) ? 1 : 0, (flags & PW_ADJ_ADD_LAMBDA) ? 1 : 0,
-                                           cf, nseg, h->d_err, ac, s);
+                                           cf, h->d_err, ac, s);
         if (e != cudaSuccess) return cuda_fail(e, "adjoint kernel launch");
         h->last_kernel = 2;
         return PW_OK;
@@ -1095,7 +1157,7 @@ pw_status_t pw_fill_halo_periodic(pw_handle_t h, void* f, pw_stream_t stream) {
         pw_status_t dst = check_device_ptrs(h, &p, 1);
         if (dst != PW_OK) return dst;
     }
-    cudaError_t e = launch_fill_halo(h->grid.dtype, to_dev(h->grid), f, h->num_sms,
+    cudaError_t e = launch_fill_halo(h->grid.dtype, to_dev(h->grid), &f, 1, h->num_sms,
                                      reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "halo fill launch");
     return PW_OK;

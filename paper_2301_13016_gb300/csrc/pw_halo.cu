@@ -9,8 +9,14 @@ namespace pw {
 // periodic image directly (i' = 1 + (i-1) mod nx, likewise j), which equals
 // the x-then-y two-pass swap including the corners.  Pure element copies in
 // the storage type (E = 4 or 2 bytes).
+// blockIdx.y = field: one launch for the fields of a state (three launches of
+// one field each cost 3 x 2.2 us on an idle GPU at 512^2 x 64, one 3.1 us).
+struct HaloFields {
+    void* f[3];
+};
 template <typename E>
-__global__ void fill_halo_kernel(const GridDev g, E* __restrict__ f) {
+__global__ void fill_halo_kernel(const GridDev g, const HaloFields fs) {
+    E* __restrict__ const f = reinterpret_cast<E*>(fs.f[blockIdx.y]);
     const int h = g.halo;
     const long long wx = g.nx + 2 * h;
     const long long rows = 2LL * h * wx;              // halo rows, full width
@@ -39,17 +45,20 @@ __global__ void fill_halo_kernel(const GridDev g, E* __restrict__ f) {
     }
 }
 
-cudaError_t launch_fill_halo(pw_dtype_t dt, const GridDev& g, void* f, int num_sms, cudaStream_t s) {
+cudaError_t launch_fill_halo(pw_dtype_t dt, const GridDev& g, void* const* f, int n, int num_sms, cudaStream_t s) {
     const long long per_level = 2LL * g.halo * (g.nx + 2 * g.halo) + 2LL * g.halo * g.ny;
     const long long total = per_level * g.nz;
     const int threads = 256;
     long long blocks = (total + threads - 1) / threads;
     if (blocks > (long long)num_sms * 8) blocks = (long long)num_sms * 8;
     if (blocks < 1) blocks = 1;
+    HaloFields fs{};
+    for (int q = 0; q < n; ++q) fs.f[q] = f[q];
+    const dim3 grid((unsigned)blocks, (unsigned)n);
     if (dtype_size(dt) == 4)
-        fill_halo_kernel<uint32_t><<<(unsigned)blocks, threads, 0, s>>>(g, (uint32_t*)f);
+        fill_halo_kernel<uint32_t><<<grid, threads, 0, s>>>(g, fs);
     else
-        fill_halo_kernel<uint16_t><<<(unsigned)blocks, threads, 0, s>>>(g, (uint16_t*)f);
+        fill_halo_kernel<uint16_t><<<grid, threads, 0, s>>>(g, fs);
     return cudaGetLastError();
 }
 

@@ -165,25 +165,33 @@ cudaError_t launch_adjoint(const GridDev& g, const float* u, const float* v, con
                            int accumulate, int add_lambda, int periodic, const CoefDev& cf, int num_sms,
                            cudaStream_t s);
 
-// Launch shape of the TMA adjoint: na cells per thread along x (a CTA covers
-// 32*na columns), ty rows per CTA, stages ring slots.
+// Launch shape of the TMA adjoint: na cells per thread along x, lx lanes per
+// row (a CTA covers lx*na columns), ty rows per CTA, stages ring slots.
 struct AdjConfig {
     int na = 0, ty = 0, stages = 0, nseg = 0;
+    int lx = 32;
 };
-// TMA k-march adjoint (periodic mode, FP32): maps6 = u, v, w, lsu, lsv, lsw
-// encoded for 32 lanes of c.na cells and c.ty rows; halos must be periodic.
-cudaError_t launch_adjoint_tma(const GridDev& g, int ox, const CUtensorMap* maps6, float* gu, float* gv, float* gw,
-                               float alpha, int accumulate, int add_lambda, const CoefDev& cf, int nseg, int* err,
-                               const AdjConfig& c, cudaStream_t s);
+// Where a level, row and column lie in the tensor maps of the adjoint:
+// coordinate = index + offset, for u, v, w (f) and for the sensitivities (l).
+struct AdjGeom {
+    int fx, fy, fz, lx, ly, lz;
+};
+// TMA k-march adjoint (FP32): maps6 = u, v, w, lsu, lsv, lsw for boxes of
+// 32*na + 8 (lx*na + 8) columns and ty + 2 rows; open: the full-array mode, else
+// the periodic one, in which the halos of all six hold periodic images.
+cudaError_t launch_adjoint_tma(const GridDev& g, const AdjGeom& ge, bool open, const CUtensorMap* maps6,
+                               const float* const* q6, float* const* g3, float alpha, int accumulate, int add_lambda,
+                               const CoefDev& cf, int* err, const AdjConfig& c, cudaStream_t s);
 bool adjoint_config_supported(const AdjConfig& c);
 AdjConfig adjoint_default_config();
-int adjoint_blocks_per_sm(const AdjConfig& c);
+int adjoint_blocks_per_sm(const AdjConfig& c, bool open);
 
 // Blocks of the TMA kernel resident per SM for a config (0 if it cannot launch).
 int tma_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c);    // source terms
 int step_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c);   // fused steps
 
-cudaError_t launch_fill_halo(pw_dtype_t dt, const GridDev& g, void* f, int num_sms, cudaStream_t s);
+// Periodic images in the lateral halos of n fields (n <= 3), one launch.
+cudaError_t launch_fill_halo(pw_dtype_t dt, const GridDev& g, void* const* f, int n, int num_sms, cudaStream_t s);
 
 // Bounded-wait self-test (see pw_selftest_wait_timeout).
 cudaError_t launch_selftest_wait(uint64_t limit_ns, int* err, cudaStream_t s);
@@ -252,6 +260,10 @@ bool is_device_ptr(const void* p, int device);
 #endif
 pw_status_t encode_tensor_map(const pw_grid_t& g, const void* ptr, int lx, int ty, CUtensorMap* out, int nc = 4,
                               int l2_promotion = PW_TMA_L2_PROMOTION);
+// A map of levels x rows x columns dims[2] x dims[1] x dims[0] from `base` (a
+// 16-byte aligned address inside a field), pitches of g.
+pw_status_t encode_tensor_map_dims(const pw_grid_t& g, const void* base, const long long (&dims)[3], int box_w,
+                                   int box_h, CUtensorMap* out, int l2_promotion = PW_TMA_L2_PROMOTION);
 // Same with an explicit box (box_w elements along x, box_h rows).
 pw_status_t encode_tensor_map_box(const pw_grid_t& g, const void* ptr, int box_w, int box_h, CUtensorMap* out,
                                   int l2_promotion = PW_TMA_L2_PROMOTION);
