@@ -302,12 +302,14 @@ pw_status_t pw_step_to(pw_handle_t h, const void *u, const void *v, const void *
  * output cells wrap around, and g is the sensitivity with respect to the
  * interior values (the halo contributions folded onto their images); g is
  * written on the interior only.  Cells of g not listed are not written.
- * In periodic mode, when the layout and pointers qualify for the TMA
- * kernels (and pw_set_kernel did not ask for the generic one), the TMA
- * k-march adjoint runs and the lateral halos of lsu, lsv, lsw are first
- * overwritten with their periodic images (their halo values carry no
- * meaning in this mode).  Otherwise the generic gather kernel runs; it skips
- * a term whose sensitivity is exactly 0.
+ * When the layout and pointers qualify for the TMA kernels (and
+ * pw_set_kernel did not ask for the generic one) the TMA k-march adjoint runs:
+ * in periodic mode for widths that are a multiple of 4, the lateral halos of
+ * lsu, lsv, lsw being first overwritten with their periodic images (their halo
+ * values carry no meaning in this mode); without PW_ADJ_PERIODIC for any width,
+ * unless pw_set_adjoint_config fixed a shape.  Otherwise the generic gather
+ * kernel runs.  Without PW_ADJ_PERIODIC, and in the generic kernel, a term
+ * whose sensitivity is exactly 0 is skipped.
  * FP32 storage only (PW_ERR_UNSUPPORTED otherwise).  g must not alias any
  * input.  pw_last_kernel reports 1 (generic) or 2 (TMA).
  */
@@ -316,16 +318,18 @@ pw_status_t pw_adjoint(pw_handle_t h, const void *u, const void *v, const void *
                        void *gu, void *gv, void *gw, float alpha, int32_t flags, pw_stream_t stream);
 
 /*
- * Launch shape of the TMA adjoint on this handle (0 = automatic, field by
- * field): cells = consecutive cells a thread owns along x (a CTA covers
- * 32*cells columns), ty = rows per CTA (one warp each), stages = ring slots
- * of the six planes (levels k-1, k, k+1 resident, the rest in flight), nseg =
- * CTAs along z (1..nz; automatic: the count that best fills the last wave of
- * CTAs, segments of >= 8 levels).  Instantiated (cells, ty, stages): (4,5,4)
- * (4,4,4) (4,6,4) (2,4,4) (2,5,4) (2,6,4) (2,8,4) (2,8,3); others give
- * PW_ERR_UNSUPPORTED, a negative value or nseg > nz PW_ERR_ARG.  Each cell's
- * arithmetic is the same in every shape.  pw_get_adjoint_config: out =
- * {cells, ty, stages, nseg} that the next TMA adjoint call will use.
+ * Launch shape of the periodic TMA adjoint on this handle (0 = automatic,
+ * field by field): cells = consecutive cells a thread owns along x, ty = rows
+ * per CTA, stages = ring slots of the six planes (levels k, k+1 resident, the
+ * rest in flight), nseg = CTAs along z (1..nz; automatic: the count estimated
+ * to fill the GPU best, segments of >= 4 levels; a segment never exceeds 126
+ * levels).  Instantiated (cells, ty, stages): (4,5,4) (4,4,4) (4,6,4) (2,4,4)
+ * (2,5,4) (2,6,4) (2,8,4) (2,8,3), a CTA covering 32*cells columns with one
+ * warp per row; others give PW_ERR_UNSUPPORTED, a negative value or nseg > nz
+ * PW_ERR_ARG.  Automatic: (4,6,4), and from 2^18 cells up 4 cells x 8 rows with
+ * 3 slots and 64 columns a CTA.  Each cell's arithmetic is the same in every
+ * shape.  pw_get_adjoint_config: out = {cells, ty, stages, nseg} that the next
+ * periodic TMA adjoint call will use.
  */
 pw_status_t pw_set_adjoint_config(pw_handle_t h, int32_t cells, int32_t ty, int32_t stages, int32_t nseg);
 pw_status_t pw_get_adjoint_config(pw_handle_t h, int32_t out[4]);

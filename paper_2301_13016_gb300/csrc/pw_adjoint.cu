@@ -191,8 +191,10 @@ __global__ void adjoint_gather_kernel(const GridDev g, const AdjArgs a, const Co
 // loads 16 rows of its vectors from shared memory instead of 30 (the 8 rows
 // read as level K+1 are carried to be level K).
 //
-// The shared-memory pipe is what bounds it (a 16-byte row load takes 4
-// wavefronts): 512^2 x 64 periodic 152 us a launch with the 30-row gather.
+// What bounds it: HBM at 2048^2 x 64 (166 Gcell/s, 0.88 of 36 B a cell), below
+// that the last wave and the latency of a level.  Periodic 512^2 / 1024^2 /
+// 2048^2 x 64, us a call: 128 / 435 / 1616, with the 30-row gather 163 / 554 /
+// 2099; open 384 x 320 x 64: 69, with the gather from global memory 978.
 //
 // Sensitivities count at the scheme's outputs only: interior columns (or their
 // periodic images), levels 2..nz for lsu, lsv and 2..nz-1 for lsw.  Their
@@ -226,7 +228,7 @@ struct AdjLayout {
     // coefficients {tzc1, tzc2, tzd1, tzd2} of levels kb-1..ke+1 of the CTA's k
     // segment, one float4 per level (the host keeps a segment within MAX_SEG
     // levels; OPEN within MAX_SEG_OPEN, the bits of its mask of levels to redo)
-    static constexpr int MAX_SEG = 254, MAX_SEG_OPEN = 64;
+    static constexpr int MAX_SEG = 126, MAX_SEG_OPEN = 64;
     static constexpr size_t CTZ_OFF = (((size_t)S * STAGE * 4 + S * sizeof(uint64_t) + 16 + 15) / 16) * 16;
     static constexpr size_t SMEM = CTZ_OFF + (size_t)(MAX_SEG + 2) * sizeof(float4);
 };
@@ -377,7 +379,8 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
                 }
             };
             // the value left (m) and right (p) of the thread's vector: from the
-            // neighbouring lane, at the row's ends from the staged row
+            // neighbouring lane, at the row's ends from the staged row (every
+            // lane loading it: 1652 -> 1759 us at 2048^2 x 64)
             auto nm = [&](const float* P, int f, int dj, const float (&x)[NA]) {
                 float t = __shfl_up_sync(FULL, x[NA - 1], 1, LX);
                 if (xl == 0) t = P[f * L::FIELD + dj * L::BW - 1];
@@ -601,7 +604,8 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
     bool aborted = false;
     int K = pb;
     for (; K <= ke && (K == pb || K < 3) && !aborted; ++K) aborted = !level(K, Gen{});
-#pragma unroll 1
+    constexpr int kUnroll = OPEN ? 2 : 1;   // (2: open 69.3 -> 67.9 us at 384 x 320 x 64, periodic 1616 -> 1627 at 2048^2)
+#pragma unroll kUnroll
     for (; K <= min(ke, nz - 2) && !aborted; ++K) aborted = !level(K, Fast{});
     for (; K <= ke && !aborted; ++K) aborted = !level(K, Gen{});
     if (aborted && tid == 0) {
@@ -627,9 +631,12 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
 }
 
 // Launch shapes: the ones pw_set_adjoint_config takes (32 lanes per row,
-// periodic mode), and the automatic ones (cells, lanes, rows, slots).
+// periodic mode), and the automatic one (cells, lanes, rows, slots): four CTAs
+// of 4 warps per SM.  Periodic 512^2 / 1024^2 / 2048^2 x 64 and open 384 x 320 x 64:
+// 128 / 435 / 1616 / 69 us, 32 lanes x 8 rows (two CTAs of 8 warps) 129 / 445 / 1652 /
+// 85, 16 x 16 130 / 449 / 1678 / 71; at 168 registers 32 x 8 takes 154 / 539 / 2051 / 78.
 #define PW_ADJ_CONFIGS(X) X(4, 5, 4) X(4, 4, 4) X(4, 6, 4) X(2, 4, 4) X(2, 5, 4) X(2, 6, 4) X(2, 8, 4) X(2, 8, 3)
-#define PW_ADJ_AUTO(X) X(4, 32, 8, 3) X(4, 16, 16, 3)
+#define PW_ADJ_AUTO(X) X(4, 16, 8, 3)
 
 AdjConfig adjoint_default_config() { return AdjConfig{4, 6, 4, 0}; }
 

@@ -633,10 +633,10 @@ static Step2Config choose_step2(pw_handle_t h) {
 }
 
 // Launch shape of the TMA adjoint (periodic or open mode): each field the user
-// fixed, else 4 cells x 6 rows with 4 slots for grids below kShapeMinCells, and
-// above 32 lanes x 8 rows or 16 lanes x 16 rows with 3 slots; k segments
-// (automatic) of >= 4 levels.  Shape and segments as for the k-march: the
-// lowest estimated time, a segment's start costing 2.5 levels (two planes
+// fixed, else 32 lanes x 4 cells x 6 rows with 4 slots for periodic grids below
+// kShapeMinCells, and 16 lanes x 4 cells x 8 rows with 3 slots otherwise; k
+// segments (automatic) of >= 4 levels, the count with the lowest estimated
+// time as for the k-march, a segment's start costing 2.5 levels (two planes
 // more than its levels, the priming level).
 static AdjConfig choose_adjoint(pw_handle_t h, bool open) {
     AdjConfig& cache = h->adj_auto[open ? 1 : 0];
@@ -644,35 +644,27 @@ static AdjConfig choose_adjoint(pw_handle_t h, bool open) {
     const AdjConfig d = adjoint_default_config();
     const AdjConfig& u = h->adj_user;
     const pw_grid_t& gr = h->grid;
-    AdjConfig cand[2] = {AdjConfig{u.na ? u.na : d.na, u.ty ? u.ty : d.ty, u.stages ? u.stages : d.stages, 0, 32}};
-    int nc = 1;
-    if (open || (!u.na && !u.ty && !u.stages && (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells)) {
-        cand[0] = AdjConfig{4, 8, 3, 0, 32};
-        cand[1] = AdjConfig{4, 16, 3, 0, 16};
-        nc = 2;
-    }
-    AdjConfig best = cand[0];
-    double lowest = 0.0;
-    const int wx = open ? gr.nx + 5 : gr.nx, wy = open ? gr.ny + 2 : gr.ny;
-    for (int q = 0; q < nc; ++q) {
-        AdjConfig c = cand[q];
-        const int tx = c.lx * c.na;
+    AdjConfig c{u.na ? u.na : d.na, u.ty ? u.ty : d.ty, u.stages ? u.stages : d.stages, u.nseg, 32};
+    if (open || (!u.na && !u.ty && !u.stages && (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells))
+        c = AdjConfig{4, 8, 3, u.nseg, 16};
+    if (!c.nseg) {
+        const int wx = open ? gr.nx + 5 : gr.nx, wy = open ? gr.ny + 2 : gr.ny, tx = c.lx * c.na;
         const long long tiles = (long long)((wx + tx - 1) / tx) * ((wy + c.ty - 1) / c.ty);
         const int bps = std::max(1, adjoint_blocks_per_sm(c, open));
         const long long slots = (long long)h->num_sms * bps;
-        const int lo = u.nseg ? u.nseg : 1, hi = u.nseg ? u.nseg : std::max(1, gr.nz / 4);
-        for (c.nseg = lo; c.nseg <= hi; ++c.nseg) {
-            const long long full = tiles * c.nseg / slots, rem = tiles * c.nseg - full * slots;
+        double lowest = 0.0;
+        for (int n = 1; n == 1 || gr.nz / n >= 4; ++n) {
+            const long long full = tiles * n / slots, rem = tiles * n - full * slots;
             const double last = rem ? 0.6 + 0.4 * (double)((rem + h->num_sms - 1) / h->num_sms) / bps : 0.0;
-            const double cost = ((gr.nz + c.nseg - 1) / c.nseg + 2.5) * ((double)full + last) * bps * tx * c.ty;
+            const double cost = ((gr.nz + n - 1) / n + 2.5) * ((double)full + last);
             if (lowest > 0.0 && !(cost < 0.985 * lowest)) continue;
             lowest = cost;
-            best = c;
+            c.nseg = n;
         }
     }
-    if (best.nseg > gr.nz) best.nseg = gr.nz;
-    cache = best;
-    return best;
+    if (c.nseg > gr.nz) c.nseg = gr.nz;
+    cache = c;
+    return c;
 }
 
 pw_status_t pw_set_adjoint_config(pw_handle_t h, int32_t cells, int32_t ty, int32_t stages, int32_t nseg) {
