@@ -394,7 +394,7 @@ pw_status_t pw_weighted_dot_noalloc(pw_handle_t h, const void *a, float sa, cons
  * coefficients (one dtype for all), in one persistent launch replayed from a
  * CUDA graph.  The paper scales its design by decomposing the problem into
  * independent compute units that each own part of the grid (Sec. 5); here a
- * unit is a whole grid and every (grid, tile) pair is a work item, taken
+ * unit is a whole grid and every (grid, tile) pair, or (grid, tile, k segment), is a work item, taken
  * from an atomic counter by one k-march CTA per SM slot: the deepest grids
  * first, each grid's tiles together in raster order.
  * Every grid's layout must qualify for the k-march kernel (pw_grid_default
@@ -403,9 +403,13 @@ pw_status_t pw_weighted_dot_noalloc(pw_handle_t h, const void *a, float sa, cons
 typedef struct pw_batch_s *pw_batch_t;
 
 /* Create a batch: grids[n] and coeffs[n] (HOST arrays, copied).  Allocates
- * the device tables and the work list; the tile shape starts at (lanes, 4, 4,
- * 1) for FP32 and (lanes, 8, 4, 2) for 16-bit storage, lanes = 16 when the
- * cells lie mostly in grids narrower than 256 columns, else 32. */
+ * the device tables and the work list; the tile shape (lanes_x, cells, ty,
+ * rows_per_thread) starts at (16, 4, 16, 1) for FP32 and (8, 8, 16, 3) for
+ * 16-bit storage, tiles of 64 columns, unless the cells lie mostly in
+ * grids of 512 columns and more: then at (32, 4, 8, 1), resp. (16, 8, 8, 3).  A
+ * work item is a tile's whole column of levels, or, where few items would
+ * leave the GPU waiting for the last ones, a k segment of it (at least 8
+ * levels). */
 pw_status_t pw_batch_create(int32_t n, const pw_grid_t *grids, const pw_coeffs_t *coeffs,
                             pw_batch_t *out);
 

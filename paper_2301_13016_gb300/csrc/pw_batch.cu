@@ -256,6 +256,13 @@ static TilePlan tile_plan(const pw_grid_t& g, const TmaConfig& c, const TmaConfi
     return p;
 }
 
+// A grid's k segments when none should be longer than `longest` levels, each
+// at least kBatchMinSeg long.
+constexpr int kBatchMinSeg = 8;
+static int batch_segments(int nz, int longest) {
+    return std::max(1, std::min((nz + longest - 1) / longest, nz / kBatchMinSeg));
+}
+
 }  // namespace pw
 
 using namespace pw;
@@ -277,6 +284,7 @@ struct pw_batch_s {
     BatchGridDev* h_grids = nullptr;   // pinned staging
     CUtensorMap* h_maps = nullptr;
     std::vector<int2> items;
+    std::vector<int> nseg;             // k segments of each grid in the work list
     long long cells = 0;
     TmaConfig cfg{32, 4, 4, 1};
     bool narrow_on = true;  // narrow last columns where cfg has a narrow partner
@@ -301,37 +309,87 @@ static void drop_graph(pw_batch_t b) {
     b->graph = nullptr;
 }
 
+// Resident CTAs per SM of a shape's kernel (0 with *e set if it cannot run).
+static int batch_bps(pw_dtype_t dt, const TmaConfig& c, bool dual, cudaError_t* e) {
+    int bps = 0;
+    Scales one{{1.f, 1.f, 1.f}, {1.f, 1.f, 1.f}};
+    *e = batch_dispatch(dt, c, dual, true, &bps, nullptr, nullptr, nullptr, 0, nullptr, one, nullptr, 0, nullptr);
+    if (*e == cudaSuccess && bps < 1) *e = cudaErrorInvalidConfiguration;
+    return *e == cudaSuccess ? bps : 0;
+}
+
+// The longest k segment (levels) a batch's work list should have, and the
+// estimated time with it (in levels of one cell per SM).  A whole column per
+// item is the least work: an item starts in the time of about 2.5 levels, two
+// planes more than its levels and the first copies.  But an item is also a
+// serial chain, and with few of them the GPU waits for the last ones (20 grids
+// of up to 128^2: 340 items for 456 CTAs, every one of them 32 to 128 levels
+// long).  So the columns are cut where that is estimated to be faster:
+//     work / SMs + 0.4 of a segment on a full SM, and at least one segment
+//     on an SM with few CTAs (0.6 of the full SM's level time).
+// GB300, us a call, whole columns / cut: 30 grids of up to 256^2 (42 M cells) FP16
+// 205 / 184, 6 of up to 384^2 (21 M cells) FP32 138 / 104, BF16 185 / 96; the 96
+// grids of 347 M cells keep whole columns.
+static double batch_plan(const pw_batch_s* b, const TmaConfig& cfg, const TmaConfig* ncfg, int bps, int* longest) {
+    int most = 0;
+    for (const auto& g : b->grids) most = std::max(most, (int)g.nz);
+    const double level = (double)bps * cfg.nc * cfg.lx * cfg.ty;   // cells an SM marches together
+    double best = 0.0;
+    *longest = most;
+    for (int len = most; len >= kBatchMinSeg; len = len * 7 / 8) {
+        double work = 0.0;
+        int longest_here = 0;
+        for (const auto& g : b->grids) {
+            const TilePlan p = tile_plan(g, cfg, ncfg);
+            const double area = (double)(p.tx * p.ty) * cfg.nc * cfg.lx * cfg.ty +
+                                (ncfg ? (double)p.nty * ncfg->nc * ncfg->lx * ncfg->ty : 0.0);
+            const int n = batch_segments(g.nz, len);
+            work += area * (g.nz + 2.5 * n);
+            longest_here = std::max(longest_here, (g.nz + n - 1) / n);
+        }
+        const double chain = (longest_here + 2.5) * level;
+        const double cost = std::max(work / b->num_sms + 0.4 * chain, 0.6 * chain);
+        if (best > 0.0 && !(cost < 0.97 * best)) continue;
+        best = cost;
+        *longest = len;
+    }
+    return best;
+}
+
 // Work items for the current tile shape.
-// Work order: the deepest grids first (nz), each grid's tiles together
-// in raster order (x fastest), so a tile's neighbours start at about the same
-// time and their shared halo rows and columns come from L2.  Measured on the
-// 512-grid batch: 222 Gcell/s, against 212 when the tile width was part of
-// the cost (a grid's ragged last column then ran with other grids' ones) and
-// 218 with y fastest.
+// Work order: the longest k segments first (for whole columns: the deepest
+// grids), each grid's tiles of a segment together in raster order (x fastest),
+// so a tile's neighbours start at about the same time and their shared halo
+// rows and columns come from L2.  Measured on the 512-grid batch: 222 Gcell/s,
+// against 212 when the tile width was part of the cost (a grid's ragged last
+// column then ran with other grids' ones) and 218 with y fastest.
 // The work list of shape `cfg` is built and uploaded first and the batch
 // switched to it only when everything succeeded: on failure the batch keeps
 // its previous shape, work list and captured graph.
 static pw_status_t build_items(pw_batch_t b, const TmaConfig& cfg, int ctas_per_sm, bool narrow_on) {
     TmaConfig ncfg{0, 0, 0, 1};
     const bool dual = narrow_on && narrow_partner(cfg, b->dtype, &ncfg);
+    cudaError_t e = cudaSuccess;
+    const int bps = batch_bps(b->dtype, cfg, dual, &e);
+    if (e != cudaSuccess) return internal_cuda_fail(e, "batch kernel occupancy");
+    const int per_sm = ctas_per_sm ? std::min(ctas_per_sm, bps) : bps;
+    int longest = 0;
+    batch_plan(b, cfg, dual ? &ncfg : nullptr, per_sm, &longest);
     struct Item {
         int grid, tile;
         long long cost;
     };
     std::vector<Item> v;
+    std::vector<int> nseg(b->n);
     for (int q = 0; q < b->n; ++q) {
         const TilePlan p = tile_plan(b->grids[q], cfg, dual ? &ncfg : nullptr);
-        for (int t = 0; t < p.tx * p.ty + p.nty; ++t) v.push_back({q, t, (long long)b->grids[q].nz});
+        const int nz = b->grids[q].nz, n = batch_segments(nz, longest), tiles = p.tx * p.ty + p.nty;
+        nseg[q] = n;
+        for (int t = 0; t < n * tiles; ++t) v.push_back({q, t, (long long)(nz + n - 1) / n});
     }
     std::stable_sort(v.begin(), v.end(), [](const Item& a, const Item& c) { return a.cost > c.cost; });
     std::vector<int2> items(v.size());
     for (size_t i = 0; i < v.size(); ++i) items[i] = make_int2(v[i].grid, v[i].tile);
-    int bps = 0;
-    Scales one{{1.f, 1.f, 1.f}, {1.f, 1.f, 1.f}};
-    cudaError_t e = batch_dispatch(b->dtype, cfg, dual, true, &bps, nullptr, nullptr, nullptr, 0, nullptr, one,
-                                   nullptr, 0, nullptr);
-    if (e != cudaSuccess || bps < 1)
-        return internal_cuda_fail(e == cudaSuccess ? cudaErrorInvalidConfiguration : e, "batch kernel occupancy");
     int2* d = nullptr;
     e = dev_malloc(&d, std::max<size_t>(1, items.size()) * sizeof(int2));
     if (e == cudaSuccess) e = cudaMemcpy(d, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice);
@@ -347,12 +405,12 @@ static pw_status_t build_items(pw_batch_t b, const TmaConfig& cfg, int ctas_per_
     cudaFree(b->d_items);
     b->d_items = d;
     b->items.swap(items);
+    b->nseg.swap(nseg);
     b->cfg = cfg;
     b->ncfg = ncfg;
     b->dual = dual;
     b->narrow_on = narrow_on;
     b->ctas_per_sm = ctas_per_sm;
-    const int per_sm = ctas_per_sm ? std::min(ctas_per_sm, bps) : bps;
     b->ctas = PW_BATCH_GRID_LAUNCH ? std::max<int>(1, (int)b->items.size()) : b->num_sms * per_sm;
     b->items_ok = true;
     b->tables_ok = false;
@@ -369,10 +427,11 @@ pw_status_t pw_batch_create(int32_t n, const pw_grid_t* grids, const pw_coeffs_t
     if (!b) return bfail(PW_ERR_OOM, "host allocation of the batch failed");
     b->n = n;
     b->dtype = grids[0].dtype;
-    // Starting tile (the autotuner refines it): 16-lane tiles when the cells
-    // lie mostly in grids narrower than 256 columns, and for 16-bit storage
-    // the packed two-row tile of 8 rows.  On the 512-grid batch (widths
-    // 32..384): FP32 7.9 ms against 8.6 for 32 x 4; BF16 6.7 against 8.8.
+    // Starting tile (the autotuner refines it), 64 columns wide unless the cells
+    // lie mostly in grids of 512 columns and more (then 128, fewer halo columns);
+    // narrow last columns either way.  96 grids of widths 32..384, 347 M cells, FP32: 64 x 16
+    // 1451 us, 64 x 8 1527, 64 x 4 1597; 64 such grids in BF16, x pairs of 8 cells:
+    // 64 x 16 753, 128 x 8 776, two rows per thread on 64 x 8 1011.
     {
         double cells = 0.0, wx = 0.0;
         for (int q = 0; q < n; ++q) {
@@ -380,11 +439,11 @@ pw_status_t pw_batch_create(int32_t n, const pw_grid_t* grids, const pw_coeffs_t
             cells += c;
             wx += c * grids[q].nx;
         }
-        b->cfg.lx = (cells > 0.0 && wx / cells < 256.0) ? 16 : 32;
-        if (b->dtype != PW_F32) {
-            b->cfg.ty = 8;
-            b->cfg.rp = 2;
-        }
+        const bool half = b->dtype != PW_F32, slim = cells > 0.0 && wx / cells < 512.0;
+        b->cfg.nc = half ? 8 : 4;
+        b->cfg.xp = half ? 1 : 0;
+        b->cfg.lx = (slim ? 64 : 128) / b->cfg.nc;
+        b->cfg.ty = slim ? 16 : 8;
     }
     size_t tz_total = 0;
     for (int q = 0; q < n; ++q) {
@@ -568,7 +627,7 @@ pw_status_t pw_batch_tendencies(pw_batch_t b, const void* const* u, const void* 
             r.tiles_y = tp.ty;
             r.ntiles_y = tp.nty;
             r.nbx = tp.nbx;
-            r.nseg = 1;
+            r.nseg = b->nseg[q];
             r.tcx = b->tcx[q];
             r.tcy = b->tcy[q];
             r.tz = b->d_tz + b->tz_off[q];
