@@ -306,10 +306,12 @@ pw_status_t pw_step_to(pw_handle_t h, const void *u, const void *v, const void *
  * pw_set_kernel did not ask for the generic one) the TMA k-march adjoint runs:
  * in periodic mode for widths that are a multiple of 4, the lateral halos of
  * lsu, lsv, lsw being first overwritten with their periodic images (their halo
- * values carry no meaning in this mode); without PW_ADJ_PERIODIC for any width,
- * unless pw_set_adjoint_config fixed a shape.  Otherwise the generic gather
- * kernel runs.  Without PW_ADJ_PERIODIC, and in the generic kernel, a term
- * whose sensitivity is exactly 0 is skipped.
+ * values carry no meaning in this mode); unless pw_set_adjoint_config fixed a
+ * shape, in periodic mode for other widths (from 32 columns and 2^18 cells up;
+ * the halos of lsu, lsv, lsw are neither read nor written then) and without
+ * PW_ADJ_PERIODIC for any width.  Otherwise the generic gather kernel runs.  A
+ * term whose sensitivity is exactly 0 is skipped, but for the periodic k-march
+ * of a width that is a multiple of 4.
  * FP32 storage only (PW_ERR_UNSUPPORTED otherwise).  g must not alias any
  * input.  pw_last_kernel reports 1 (generic) or 2 (TMA).
  */

@@ -143,15 +143,32 @@ __device__ __forceinline__ void adjoint_gather_cell(const GridDev& g, const AdjA
 #undef PW_ADD
 }
 
-__global__ void adjoint_gather_kernel(const GridDev g, const AdjArgs a, const CoefDev cf) {
+// One thread per cell: every cell the mode writes, or (RING) the interior cells
+// of the first and last row and column only (nx, ny >= 3).  64 registers, so
+// that four CTAs share an SM (76 registers: 273 -> 341 us at 170 x 421 x 37).
+template <bool RING>
+__global__ void __launch_bounds__(256, 4) adjoint_gather_kernel(const GridDev g, const AdjArgs a, const CoefDev cf) {
     const int h = a.periodic ? 0 : 1;   // extra ring of cells covered in full-array mode
     const long long wx = g.nx + 2 * h, wy = g.ny + 2 * h;
-    const long long total = wx * wy * g.nz;
+    const long long per_level = RING ? 2LL * (g.nx + g.ny - 2) : wx * wy;
+    const long long total = per_level * g.nz;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
-        const int I = (int)(idx % wx) + 1 - h;
-        const int J = (int)((idx / wx) % wy) + 1 - h;
-        const int K = 1 + (int)(idx / (wx * wy));
+        int I, J;
+        const int K = 1 + (int)(idx / per_level);
+        if (RING) {
+            const int t = (int)(idx % per_level);
+            if (t < 2 * g.nx) {
+                I = 1 + t % g.nx;
+                J = t < g.nx ? 1 : g.ny;
+            } else {
+                I = (t & 1) ? g.nx : 1;
+                J = 2 + ((t - 2 * g.nx) >> 1);
+            }
+        } else {
+            I = (int)(idx % wx) + 1 - h;
+            J = (int)((idx / wx) % wy) + 1 - h;
+        }
         float ru, rv, rw;
         adjoint_gather_cell(g, a, cf, K, J, I, ru, rv, rw);
         const long long c = g.origin + (long long)K * g.pk + (long long)J * g.pj + I;
@@ -200,14 +217,20 @@ __global__ void adjoint_gather_kernel(const GridDev g, const AdjArgs a, const Co
 // periodic images), levels 2..nz for lsu, lsv and 2..nz-1 for lsw.  Their
 // tensor maps cover just those, so the copy engine's zero fill masks the rest.
 //
-// OPEN: the full-array mode (every cell of the interior and its one-cell halo,
-// halo values of u, v, w as independent inputs): tiles start at column -3
-// (16-byte aligned) and row 0, the maps of l cover the interior, the maps of
-// u, v, w columns -3..nx+1 and rows 0..ny+1.  This mode skips a term whose
-// sensitivity is exactly 0, which matters where the field is not finite: a
-// level of a thread whose result is not finite is not stored but redone cell
-// by cell by adjoint_gather_cell after the march (any field value that is
-// not finite makes the result so, zero sensitivity or not).
+// The full-array mode (every cell of the interior and its one-cell halo, halo
+// values of u, v, w as independent inputs): tiles start at column -3 (16-byte
+// aligned) and row 0, the maps of l cover the interior, the maps of u, v, w
+// columns -3..nx+1 and rows 0..ny+1.  The periodic mode of a width that is no
+// multiple of 4: the march writes the cells that touch no image (columns
+// 2..nx-1, rows 2..ny-1; the maps of l cover the interior), and a second
+// launch gathers the ring of cells around them, so the halos of l are neither
+// read nor written there (511 x 512 x 64: 182 us, with the gather kernel alone 1785).
+//
+// CHECKED (both of these): a term whose sensitivity is exactly 0 is skipped,
+// which matters where the field is not finite: a level of a thread whose result
+// is not finite is not stored but redone cell by cell by adjoint_gather_cell
+// after the march (any field value that is not finite makes the result so,
+// zero sensitivity or not).
 constexpr int kAdjPAD = 4;                       // 16-byte granule of FP32
 
 template <int NA, int LX, int TY, int S>
@@ -227,8 +250,8 @@ struct AdjLayout {
     // the ring, one mbarrier per slot, 4 flag words, then the vertical
     // coefficients {tzc1, tzc2, tzd1, tzd2} of levels kb-1..ke+1 of the CTA's k
     // segment, one float4 per level (the host keeps a segment within MAX_SEG
-    // levels; OPEN within MAX_SEG_OPEN, the bits of its mask of levels to redo)
-    static constexpr int MAX_SEG = 126, MAX_SEG_OPEN = 64;
+    // levels; CHECKED within MAX_SEG_CHECKED, the bits of its mask of levels to redo)
+    static constexpr int MAX_SEG = 126, MAX_SEG_CHECKED = 64;
     static constexpr size_t CTZ_OFF = (((size_t)S * STAGE * 4 + S * sizeof(uint64_t) + 16 + 15) / 16) * 16;
     static constexpr size_t SMEM = CTZ_OFF + (size_t)(MAX_SEG + 2) * sizeof(float4);
 };
@@ -283,7 +306,7 @@ constexpr int adj_min_blocks() {
     return m < 1 ? 1 : m;
 }
 
-template <int NA, int LX, int TY, int S, bool OPEN>
+template <int NA, int LX, int TY, int S, bool CHECKED>
 __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_blocks<NA, LX, TY, S>()))
     adjoint_march_kernel(const __grid_constant__ AdjMaps maps, const AdjArgs a, const GridDev g, const AdjGeom ge,
                          const int nseg, const CoefDev cf, int* __restrict__ err) {
@@ -301,8 +324,8 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
     const int ke = (int)(((long long)(blockIdx.z + 1) * nz) / nseg);
     if (ke < kb) return;
     const int pb = max(kb - 1, 1), pe = min(ke + 1, nz), np = pe - pb + 1;
-    const int i_tile = (OPEN ? -3 : 1) + L::TX * blockIdx.x;   // first column and row of the tile
-    const int j_tile = (OPEN ? 0 : 1) + TY * blockIdx.y;
+    const int i_tile = (CHECKED ? ge.i0 : 1) + L::TX * blockIdx.x;   // first column and row of the tile
+    const int j_tile = (CHECKED ? ge.j0 : 1) + TY * blockIdx.y;
 
     auto issue = [&](int p) {
         const int s = p % S, k = pb + p;
@@ -340,16 +363,16 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
     const float tcx = cf.tcx, tcy = cf.tcy;
     const int J = j_tile + ty, I0 = i_tile + NA * xl;
     const int c0 = (ty + 1) * L::BW + kAdjPAD + NA * xl;   // the thread's vector in a staged field
-    const int ilo = OPEN ? 0 : 1, ihi = OPEN ? g.nx + 1 : g.nx;
-    const bool valid = J <= (OPEN ? g.ny + 1 : g.ny) && I0 <= ihi && (!OPEN || I0 + NA > 0);
+    const int ilo = CHECKED ? ge.ilo : 1, ihi = CHECKED ? ge.ihi : g.nx;
+    const bool valid = (!CHECKED || (J >= ge.jlo && I0 + NA > ilo)) && J <= (CHECKED ? ge.jhi : g.ny) && I0 <= ihi;
     const bool whole = I0 >= ilo && I0 + NA - 1 <= ihi;
     // sensitivities as the caller gave them: staged where they count, else in memory
-    const bool staged = !OPEN || (J >= 1 && J <= g.ny && I0 >= 1 && I0 + NA - 1 <= g.nx);
-    const bool left = OPEN && I0 < 0;   // columns -3..-1 hold padding
+    const bool staged = !CHECKED || (J >= 1 && J <= g.ny && I0 >= 1 && I0 + NA - 1 <= g.nx);
+    const bool left = CHECKED && I0 < 0;   // columns -3..-1 hold padding
     const long long row_off = g.origin + (long long)J * g.pj + I0;
     const unsigned FULL = 0xffffffffu;
     int waited = 0;
-    unsigned long long redo = 0;   // OPEN: levels kb + bit whose result was not finite
+    unsigned long long redo = 0;   // CHECKED: levels kb + bit whose result was not finite
 
     AdjRegs<NA> st;
 #pragma unroll
@@ -484,7 +507,7 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
                     if (up) r0[c] = fmaf(c1p * nx.lu[c], PX[c], r0[c]);
                 }
                 finish(a.gu, a.lu, st.lu, r0);
-                if (!OPEN) store(a.gu, r0);
+                if (!CHECKED) store(a.gu, r0);
                 // ---- gv: v in su (as b, d), in sv (as a, b, d), in sw (as b, d)
                 float uq[NA], vq[NA], lvq[NA];
                 row(P0, U, 1, uq);
@@ -508,7 +531,7 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
                     Q = Qn;
                 }
                 finish(a.gv, a.lv, st.lv, r1);
-                if (!OPEN) store(a.gv, r1);
+                if (!CHECKED) store(a.gv, r1);
                 // ---- gw: w in su, sv (as b, d), in sw (as a, b, d)
                 if (up) {
                     row(P1, U, 0, nx.u);
@@ -554,7 +577,7 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
                     }
                 }
                 finish(a.gw, a.lw, st.lw, r2);
-                if (!OPEN) {
+                if (!CHECKED) {
                     store(a.gw, r2);
                 } else {
                     float t = 0.f;   // stays 0 while every result is finite
@@ -604,7 +627,7 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
     bool aborted = false;
     int K = pb;
     for (; K <= ke && (K == pb || K < 3) && !aborted; ++K) aborted = !level(K, Gen{});
-    constexpr int kUnroll = OPEN ? 2 : 1;   // (2: open 69.3 -> 67.9 us at 384 x 320 x 64, periodic 1616 -> 1627 at 2048^2)
+    constexpr int kUnroll = CHECKED ? 2 : 1;   // (2: open 69.3 -> 67.9 us at 384 x 320 x 64, periodic 1616 -> 1627 at 2048^2)
 #pragma unroll kUnroll
     for (; K <= min(ke, nz - 2) && !aborted; ++K) aborted = !level(K, Fast{});
     for (; K <= ke && !aborted; ++K) aborted = !level(K, Gen{});
@@ -614,7 +637,7 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
         for (int p = waited; p < issued; ++p)
             if (!mbar_wait_bounded(&bars[p % S], (uint32_t)((p / S) & 1), kDrainLimitNs)) break;
     }
-    if constexpr (OPEN) {
+    if constexpr (CHECKED) {
         while (redo && !aborted) {
             const int Kr = kb + __ffsll((long long)redo) - 1;
             redo &= redo - 1;
@@ -648,52 +671,59 @@ bool adjoint_config_supported(const AdjConfig& c) {
     return false;
 }
 
-template <int NA, int LX, int TY, int S, bool OPEN>
+template <int NA, int LX, int TY, int S, bool CHECKED>
 static cudaError_t adj_inst(const AdjConfig& c, int* bps, const GridDev& g, const AdjGeom& ge, const AdjMaps& m,
                             const AdjArgs& a, const CoefDev& cf, int* err, cudaStream_t s) {
     using L = AdjLayout<NA, LX, TY, S>;
-    auto kern = adjoint_march_kernel<NA, LX, TY, S, OPEN>;
+    auto kern = adjoint_march_kernel<NA, LX, TY, S, CHECKED>;
     cudaError_t e = set_smem_attr_once(kern, (int)L::SMEM);
     if (e != cudaSuccess) return e;
     if (bps) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, kern, L::THREADS, L::SMEM);
-    constexpr int most = OPEN ? L::MAX_SEG_OPEN : L::MAX_SEG;
+    constexpr int most = CHECKED ? L::MAX_SEG_CHECKED : L::MAX_SEG;
     const int nseg = std::max(c.nseg, (g.nz + most - 1) / most);
-    const int wx = OPEN ? g.nx + 5 : g.nx, wy = OPEN ? g.ny + 2 : g.ny;        // OPEN: columns -3..nx+1, rows 0..ny+1
+    const int wx = ge.ihi - ge.i0 + 1, wy = ge.jhi - ge.j0 + 1;
     dim3 grid((wx + L::TX - 1) / L::TX, (wy + TY - 1) / TY, nseg);
     kern<<<grid, dim3(32, L::WARPS), L::SMEM, s>>>(m, a, g, ge, nseg, cf, err);
     return cudaGetLastError();
 }
 
-static cudaError_t adj_dispatch(const AdjConfig& c, bool open, int* bps, const GridDev& g, const AdjGeom& ge,
+static cudaError_t adj_dispatch(const AdjConfig& c, bool checked, int* bps, const GridDev& g, const AdjGeom& ge,
                                 const AdjMaps& m, const AdjArgs& a, const CoefDev& cf, int* err, cudaStream_t s) {
 #define PW_AA(NA_, LX_, TY_, S_)                                                                      \
     if (c.na == NA_ && c.lx == LX_ && c.ty == TY_ && c.stages == S_)                                  \
-        return open ? adj_inst<NA_, LX_, TY_, S_, true>(c, bps, g, ge, m, a, cf, err, s)              \
+        return checked ? adj_inst<NA_, LX_, TY_, S_, true>(c, bps, g, ge, m, a, cf, err, s)              \
                     : adj_inst<NA_, LX_, TY_, S_, false>(c, bps, g, ge, m, a, cf, err, s);
     PW_ADJ_AUTO(PW_AA)
 #undef PW_AA
 #define PW_AD(NA_, TY_, S_)                                                                           \
-    if (!open && c.lx == 32 && c.na == NA_ && c.ty == TY_ && c.stages == S_)                          \
+    if (!checked && c.lx == 32 && c.na == NA_ && c.ty == TY_ && c.stages == S_)                          \
         return adj_inst<NA_, 32, TY_, S_, false>(c, bps, g, ge, m, a, cf, err, s);
     PW_ADJ_CONFIGS(PW_AD)
 #undef PW_AD
     return cudaErrorInvalidConfiguration;
 }
 
-int adjoint_blocks_per_sm(const AdjConfig& c, bool open) {
+int adjoint_blocks_per_sm(const AdjConfig& c, bool checked) {
     int n = 0;
-    if (adj_dispatch(c, open, &n, GridDev{}, AdjGeom{}, AdjMaps{}, AdjArgs{}, CoefDev{}, nullptr, nullptr) != cudaSuccess)
+    if (adj_dispatch(c, checked, &n, GridDev{}, AdjGeom{}, AdjMaps{}, AdjArgs{}, CoefDev{}, nullptr, nullptr) != cudaSuccess)
         return 0;
     return n;
 }
 
-cudaError_t launch_adjoint_tma(const GridDev& g, const AdjGeom& ge, bool open, const CUtensorMap* maps6,
+cudaError_t launch_adjoint_tma(const GridDev& g, const AdjGeom& ge, AdjMode mode, const CUtensorMap* maps6,
                                const float* const* q6, float* const* g3, float alpha, int accumulate, int add_lambda,
-                               const CoefDev& cf, int* err, const AdjConfig& c, cudaStream_t s) {
+                               const CoefDev& cf, int* err, const AdjConfig& c, int num_sms, cudaStream_t s) {
     AdjMaps m;
     for (int f = 0; f < 6; ++f) m.m[f] = maps6[f];
-    const AdjArgs a{q6[0], q6[1], q6[2], q6[3], q6[4], q6[5], g3[0], g3[1], g3[2], alpha, accumulate, add_lambda, !open};
-    return adj_dispatch(c, open, nullptr, g, ge, m, a, cf, err, s);
+    const AdjArgs a{q6[0], q6[1], q6[2], q6[3], q6[4], q6[5], g3[0], g3[1], g3[2], alpha, accumulate, add_lambda,
+                    mode != ADJ_OPEN};
+    cudaError_t e = adj_dispatch(c, mode != ADJ_PERIODIC, nullptr, g, ge, m, a, cf, err, s);
+    if (e == cudaSuccess && mode == ADJ_PERIODIC_ANY) {
+        const long long ring = 2LL * (g.nx + g.ny - 2) * g.nz;
+        adjoint_gather_kernel<true><<<(unsigned)std::min<long long>((ring + 255) / 256, num_sms * 16), 256, 0, s>>>(g, a, cf);
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 cudaError_t launch_adjoint(const GridDev& g, const float* u, const float* v, const float* w, const float* lu,
@@ -707,7 +737,7 @@ cudaError_t launch_adjoint(const GridDev& g, const float* u, const float* v, con
     long long blocks = (total + threads - 1) / threads;
     if (blocks > (long long)num_sms * 16) blocks = (long long)num_sms * 16;
     if (blocks < 1) blocks = 1;
-    adjoint_gather_kernel<<<(unsigned)blocks, threads, 0, s>>>(g, a, cf);
+    adjoint_gather_kernel<false><<<(unsigned)blocks, threads, 0, s>>>(g, a, cf);
     return cudaGetLastError();
 }
 

@@ -88,7 +88,7 @@ struct pw_handle_s {
     Step2Config step2_user{0, 0, 0, 0};
     Step2Config step2_auto{0, 0, 0, 0};   // ty == 0: not chosen yet
     AdjConfig adj_user{0, 0, 0, 0};       // TMA adjoint shape; 0 = automatic
-    AdjConfig adj_auto[2] = {};           // the shape in use (periodic, open mode); na == 0: not chosen yet
+    AdjConfig adj_auto[3] = {};           // the shape in use, per AdjMode; na == 0: not chosen yet
     MapCacheEntry maps[8];
     int map_next = 0;   // round-robin replacement
     // field pointers already found to be device memory of this handle's GPU
@@ -237,31 +237,34 @@ pw_status_t pw::encode_tensor_map_dims(const pw_grid_t& g, const void* base, con
 }
 
 // A tensor map of the TMA adjoint for field f of (u, v, w, lsu, lsv, lsw), and
-// where levels, rows and columns lie in such maps (AdjGeom).  Periodic mode:
-// whole rows with their halos, levels 1..nz of u, v, w, 2..nz of lsu and lsv,
-// 2..nz-1 of lsw.  Open mode: u, v, w on columns -3..nx+1 (-3 is the first
-// 16-byte boundary at or before column 0; interior rows start on one) and rows
-// 0..ny+1, the sensitivities on the interior.
-static AdjGeom adj_geom(const pw_grid_t& g, int ox, bool open) {
-    if (open) return AdjGeom{3, 0, -1, -1, -1, -2};
-    return AdjGeom{ox, g.halo - 1, -1, ox, g.halo - 1, -2};
+// where levels, rows and columns lie in such maps (AdjGeom).  u, v, w: levels
+// 1..nz of whole rows with their halos, or (open mode) of columns -3..nx+1 (-3 is
+// the first 16-byte boundary at or before column 0; interior rows start on one)
+// and rows 0..ny+1.  Sensitivities: levels 2..nz (lsw 2..nz-1) of whole rows with
+// their halos, or (the modes that do not read these) of the interior.
+static AdjGeom adj_geom(const pw_grid_t& g, int ox, AdjMode mode) {
+    if (mode == ADJ_OPEN) return AdjGeom{3, 0, -1, -1, -1, -2, -3, 0, 0, g.nx + 1, 0, g.ny + 1};
+    if (mode == ADJ_PERIODIC_ANY)
+        return AdjGeom{ox, g.halo - 1, -1, -1, -1, -2, 1, 1, 2, g.nx - 1, 2, g.ny - 1};
+    return AdjGeom{ox, g.halo - 1, -1, ox, g.halo - 1, -2, 1, 1, 1, g.nx, 1, g.ny};
 }
-static pw_status_t adj_map(pw_handle_t h, int f, const void* ptr, bool open, int ox, int box_w, int box_h,
+static pw_status_t adj_map(pw_handle_t h, int f, const void* ptr, AdjMode mode, int ox, int box_w, int box_h,
                            CUtensorMap* out) {
-    const int kind = MAP_ADJ + 2 * (f < 3 ? 0 : (f < 5 ? 1 : 2)) + (open ? 1 : 0);
+    const int kind = MAP_ADJ + 3 * (f < 3 ? 0 : (f < 5 ? 1 : 2)) + (int)mode;
     for (auto& c : h->maps)
         if (c.ptr == ptr && c.kind == kind && c.box_w == box_w && c.box_h == box_h) {
             *out = c.map;
             return PW_OK;
         }
     const pw_grid_t& g = h->grid;
-    const AdjGeom ge = adj_geom(g, ox, open);
+    const AdjGeom ge = adj_geom(g, ox, mode);
     // the map's first element: level, row and column with coordinate 0
     const long long k = f < 3 ? -ge.fz : -ge.lz, j = f < 3 ? -ge.fy : -ge.ly, i = f < 3 ? -ge.fx : -ge.lx;
     const float* base = static_cast<const float*>(ptr) + g.origin + k * g.pitch_k + j * g.pitch_j + i;
     const long long levels = f < 3 ? g.nz : (f < 5 ? g.nz - 1 : g.nz - 2);
-    const long long rows = !open ? g.ny + 2LL * g.halo : (f < 3 ? g.ny + 2 : g.ny);
-    const long long cols = !open ? ox + g.nx + g.halo + 1LL : (f < 3 ? g.nx + 5 : g.nx);
+    const bool whole = mode == ADJ_PERIODIC || (mode == ADJ_PERIODIC_ANY && f < 3);
+    const long long rows = whole ? g.ny + 2LL * g.halo : (f < 3 ? g.ny + 2 : g.ny);
+    const long long cols = whole ? ox + g.nx + g.halo + 1LL : (f < 3 ? g.nx + 5 : g.nx);
     pw_status_t st = encode_tensor_map_dims(g, base, {cols, rows, levels}, box_w, box_h, out);
     if (st != PW_OK) return st;
     MapCacheEntry& e = h->maps[h->map_next];
@@ -638,19 +641,20 @@ static Step2Config choose_step2(pw_handle_t h) {
 // segments (automatic) of >= 4 levels, the count with the lowest estimated
 // time as for the k-march, a segment's start costing 2.5 levels (two planes
 // more than its levels, the priming level).
-static AdjConfig choose_adjoint(pw_handle_t h, bool open) {
-    AdjConfig& cache = h->adj_auto[open ? 1 : 0];
+static AdjConfig choose_adjoint(pw_handle_t h, AdjMode mode) {
+    AdjConfig& cache = h->adj_auto[mode];
     if (cache.na) return cache;
     const AdjConfig d = adjoint_default_config();
     const AdjConfig& u = h->adj_user;
     const pw_grid_t& gr = h->grid;
     AdjConfig c{u.na ? u.na : d.na, u.ty ? u.ty : d.ty, u.stages ? u.stages : d.stages, u.nseg, 32};
-    if (open || (!u.na && !u.ty && !u.stages && (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells))
+    if (mode != ADJ_PERIODIC || (!u.na && !u.ty && !u.stages && (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells))
         c = AdjConfig{4, 8, 3, u.nseg, 16};
     if (!c.nseg) {
-        const int wx = open ? gr.nx + 5 : gr.nx, wy = open ? gr.ny + 2 : gr.ny, tx = c.lx * c.na;
+        const AdjGeom ge = adj_geom(gr, 0, mode);
+        const int wx = ge.ihi - ge.i0 + 1, wy = ge.jhi - ge.j0 + 1, tx = c.lx * c.na;
         const long long tiles = (long long)((wx + tx - 1) / tx) * ((wy + c.ty - 1) / c.ty);
-        const int bps = std::max(1, adjoint_blocks_per_sm(c, open));
+        const int bps = std::max(1, adjoint_blocks_per_sm(c, mode != ADJ_PERIODIC));
         const long long slots = (long long)h->num_sms * bps;
         double lowest = 0.0;
         for (int n = 1; n == 1 || gr.nz / n >= 4; ++n) {
@@ -677,13 +681,13 @@ pw_status_t pw_set_adjoint_config(pw_handle_t h, int32_t cells, int32_t ty, int3
         return fail(PW_ERR_UNSUPPORTED, "no TMA adjoint instance for cells=%d ty=%d stages=%d", c.na, c.ty,
                     c.stages);
     h->adj_user = AdjConfig{cells, ty, stages, nseg};
-    h->adj_auto[0] = h->adj_auto[1] = AdjConfig{};
+    for (auto& c : h->adj_auto) c = AdjConfig{};
     return PW_OK;
 }
 
 pw_status_t pw_get_adjoint_config(pw_handle_t h, int32_t out[4]) {
     if (!h || !out) return fail(PW_ERR_ARG, "handle or out is NULL");
-    const AdjConfig c = choose_adjoint(h, false);
+    const AdjConfig c = choose_adjoint(h, ADJ_PERIODIC);
     out[0] = c.na;
     out[1] = c.ty;
     out[2] = c.stages;
@@ -1102,30 +1106,37 @@ pw_status_t pw_adjoint(pw_handle_t h, const void* u, const void* v, const void* 
     const char* why = "";
     bool ptrs_ok = true;
     for (auto p : ins) ptrs_ok = ptrs_ok && aligned16(p);
-    const bool open = !(flags & PW_ADJ_PERIODIC);
-    const AdjConfig& au = h->adj_user;
     for (auto p : outs) ptrs_ok = ptrs_ok && aligned16(p);
-    // the open mode takes any width, with the automatic shape
-    const bool shape_ok = !open || !(au.na || au.ty || au.stages || au.nseg);
-    if (h->kernel_kind != 1 && ptrs_ok && shape_ok && tma_layout_ok(h->grid, &ox, &why, open)) {
-        const GridDev g = to_dev(h->grid);
-        if (!open) {   // the sensitivities need periodic halos too
+    // Widths that are a multiple of 4 in periodic mode; the full array at any
+    // width; and periodic ones at any width from kRagMinNx columns and
+    // kShapeMinCells cells up (the ring of cells gathered by a second launch is
+    // then a small part), both with the automatic shape.
+    const pw_grid_t& gr = h->grid;
+    const AdjConfig& au = h->adj_user;
+    const bool fixed = au.na || au.ty || au.stages || au.nseg;
+    const AdjMode mode = !(flags & PW_ADJ_PERIODIC) ? ADJ_OPEN : (gr.nx % 4 == 0 ? ADJ_PERIODIC : ADJ_PERIODIC_ANY);
+    const bool size_ok = mode != ADJ_PERIODIC_ANY || (h->kernel_kind == 0 && gr.nx >= kRagMinNx && gr.ny >= 8 &&
+                                                      (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells);
+    if (h->kernel_kind != 1 && ptrs_ok && size_ok && (mode == ADJ_PERIODIC || !fixed) &&
+        tma_layout_ok(gr, &ox, &why, mode != ADJ_PERIODIC)) {
+        const GridDev g = to_dev(gr);
+        if (mode == ADJ_PERIODIC) {   // the sensitivities need periodic halos too
             void* ls[3] = {const_cast<void*>(lsu), const_cast<void*>(lsv), const_cast<void*>(lsw)};
             cudaError_t e = launch_fill_halo(PW_F32, g, ls, 3, h->num_sms, s);
             if (e != cudaSuccess) return cuda_fail(e, "sensitivity halo fill");
         }
         CUtensorMap maps[6];
-        const AdjConfig ac = choose_adjoint(h, open);
+        const AdjConfig ac = choose_adjoint(h, mode);
         for (int q = 0; q < 6; ++q) {
-            pw_status_t st = adj_map(h, q, ins[q], open, ox, ac.lx * ac.na + 8, ac.ty + 2, &maps[q]);
+            pw_status_t st = adj_map(h, q, ins[q], mode, ox, ac.lx * ac.na + 8, ac.ty + 2, &maps[q]);
             if (st != PW_OK) return st;
         }
         const float* q6[6] = {(const float*)u,   (const float*)v,   (const float*)w,
                               (const float*)lsu, (const float*)lsv, (const float*)lsw};
         float* g3[3] = {(float*)gu, (float*)gv, (float*)gw};
-        cudaError_t e = launch_adjoint_tma(g, adj_geom(h->grid, ox, open), open, maps, q6, g3, alpha,
+        cudaError_t e = launch_adjoint_tma(g, adj_geom(gr, ox, mode), mode, maps, q6, g3, alpha,
                                            (flags & PW_ADJ_ACCUMULATE) ? 1 : 0, (flags & PW_ADJ_ADD_LAMBDA) ? 1 : 0,
-                                           cf, h->d_err, ac, s);
+                                           cf, h->d_err, ac, h->num_sms, s);
         if (e != cudaSuccess) return cuda_fail(e, "adjoint kernel launch");
         h->last_kernel = 2;
         return PW_OK;

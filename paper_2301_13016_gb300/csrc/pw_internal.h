@@ -171,20 +171,25 @@ struct AdjConfig {
     int na = 0, ty = 0, stages = 0, nseg = 0;
     int lx = 32;
 };
+// Modes of the TMA adjoint: the doubly periodic domain with periodic halos of
+// the sensitivities; the same without reading their halos, for any width; the
+// full array, for any width.
+enum AdjMode { ADJ_PERIODIC, ADJ_PERIODIC_ANY, ADJ_OPEN };
 // Where a level, row and column lie in the tensor maps of the adjoint:
-// coordinate = index + offset, for u, v, w (f) and for the sensitivities (l).
+// coordinate = index + offset, for u, v, w (f) and for the sensitivities (l);
+// the first tile's first column and row; the columns and rows written.
 struct AdjGeom {
     int fx, fy, fz, lx, ly, lz;
+    int i0, j0, ilo, ihi, jlo, jhi;
 };
 // TMA k-march adjoint (FP32): maps6 = u, v, w, lsu, lsv, lsw for boxes of
-// 32*na + 8 (lx*na + 8) columns and ty + 2 rows; open: the full-array mode, else
-// the periodic one, in which the halos of all six hold periodic images.
-cudaError_t launch_adjoint_tma(const GridDev& g, const AdjGeom& ge, bool open, const CUtensorMap* maps6,
+// lx*na + 8 columns and ty + 2 rows.
+cudaError_t launch_adjoint_tma(const GridDev& g, const AdjGeom& ge, AdjMode mode, const CUtensorMap* maps6,
                                const float* const* q6, float* const* g3, float alpha, int accumulate, int add_lambda,
-                               const CoefDev& cf, int* err, const AdjConfig& c, cudaStream_t s);
+                               const CoefDev& cf, int* err, const AdjConfig& c, int num_sms, cudaStream_t s);
 bool adjoint_config_supported(const AdjConfig& c);
 AdjConfig adjoint_default_config();
-int adjoint_blocks_per_sm(const AdjConfig& c, bool open);
+int adjoint_blocks_per_sm(const AdjConfig& c, bool checked);   // checked: every mode but ADJ_PERIODIC
 
 // Blocks of the TMA kernel resident per SM for a config (0 if it cannot launch).
 int tma_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c);    // source terms

@@ -78,6 +78,32 @@ def test_periodic_automatic_shapes_match_generic(shape):
     _close(*_both(g, f, pwlib.PW_ADJ_PERIODIC | pwlib.PW_ADJ_ACCUMULATE, base))
 
 
+# widths that are no multiple of 4: the march writes all but the outermost ring of
+# cells; the sensitivities' halos (here NaN) are neither read nor written
+@pytest.mark.parametrize("shape", [(33, 200, 40), (61, 70, 65), (126, 63, 34), (127, 64, 40), (193, 15, 100)])
+def test_periodic_any_width_matches_generic(shape):
+    g = pwlib.Grid(*shape)
+    f = _fields(g, 3, wrap=True)
+    for t in f[3:]:
+        v = g.view(t)
+        v[:, 0] = v[:, -1] = NAN
+        v[:, :, 0] = v[:, :, -1] = NAN
+    lam = [t.clone() for t in f[3:]]
+    base = _fields(g, 4, 3)
+    _close(*_both(g, f, pwlib.PW_ADJ_PERIODIC))
+    _close(*_both(g, f, pwlib.PW_ADJ_PERIODIC | pwlib.PW_ADJ_ADD_LAMBDA))
+    _close(*_both(g, f, pwlib.PW_ADJ_PERIODIC | pwlib.PW_ADJ_ACCUMULATE, base))
+    for a, b in zip(f[3:], lam):
+        assert torch.equal(a.nan_to_num(5.0), b.nan_to_num(5.0))
+    v = g.view(f[1])                                # values that are not finite under zero sensitivities
+    v[3:9, 5:11, 7:30] = INF
+    for t in f[3:]:
+        g.view(t)[2:11, 4:13, 6:32] = 0.0
+    march, generic = _both(g, f, pwlib.PW_ADJ_PERIODIC)
+    _close(march, generic)
+    assert all(np.isfinite(x).all() for x in march)
+
+
 @pytest.mark.parametrize("bad", [NAN, INF, -INF])
 @pytest.mark.parametrize("flags", [0, pwlib.PW_ADJ_ADD_LAMBDA, pwlib.PW_ADJ_ACCUMULATE])
 def test_open_mode_skips_zero_sensitivities(bad, flags):
