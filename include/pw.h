@@ -345,6 +345,18 @@ pw_status_t pw_get_adjoint_config(pw_handle_t h, int32_t out[4]);
 pw_status_t pw_fill_halo_periodic(pw_handle_t h, void *f, pw_stream_t stream);
 
 /*
+ * Copy of three fields' interiors: da = a on the interior cells of levels
+ * 1..nz and 0 in every other of its first n elements (halos, z-halo planes, row
+ * padding), likewise db and dc.  n: the elements each buffer holds, at least
+ * those of the layout (as pw_grid_default counts them, or origin +
+ * (nz+1)*pitch_k + (ny+halo)*pitch_j + nx+halo+1 for a layout of one's own).
+ * An input may be NULL (zeros) or its own output (in place); the outputs are
+ * distinct, and no output is another field's input.  One launch.
+ */
+pw_status_t pw_keep_interior(pw_handle_t h, const void *a, const void *b, const void *c, void *da, void *db,
+                             void *dc, int64_t n, pw_stream_t stream);
+
+/*
  * Validation norms in FP64 over the interior cells of levels k0..k1
  * (1 <= k0 <= k1 <= nz): for a field `test` in the handle's dtype (scaled by
  * `scale`: physical = stored*scale) and a DEVICE FP64 reference `ref` in the

@@ -20,12 +20,6 @@ import torch
 from .pw import PW_ADJ_ADD_LAMBDA, PW_ADJ_PERIODIC
 
 
-def _interior_mask(grid, device):
-    m = torch.zeros(grid.alloc_elems, dtype=torch.bool, device=device)
-    grid.view(m)[1:-1, grid.halo:grid.halo + grid.ny, grid.halo:grid.halo + grid.nx] = True
-    return m
-
-
 def _new_state(grid, device, fill=None):
     """Three fields for a state that a step pass writes: levels 1..nz with
     their lateral halos (the z-halo planes and the padding are never read;
@@ -41,13 +35,16 @@ class PWRollout(torch.autograd.Function):
             raise ValueError("PWRollout needs an FP32 grid")
         every = max(1, int(checkpoint_every))
         state = [t.detach().clone() for t in (u, v, w)]
-        for t in state:                              # periodic halos of the start state
-            handle.fill_halo_periodic(t)
         ckpts = []
+        if nsteps < 1:                               # periodic halos of the start state
+            for t in state:
+                handle.fill_halo_periodic(t)
         for n in range(int(nsteps)):
             if n % every == 0:
                 ckpts.append(state)
             nxt = _new_state(grid, u.device, fill=0.0 if n == nsteps - 1 else None)
+            if n == 0:
+                handle.step(*state, *nxt, dt, 0)     # the same, all three in one launch
             handle.step_to(*state, *nxt, dt)
             state = nxt
         if not ckpts:                                # nsteps = 0: the result is a copy of the start state
@@ -63,15 +60,12 @@ class PWRollout(torch.autograd.Function):
         saved = ctx.saved_tensors
         ckpts = [saved[3 * i:3 * i + 3] for i in range(len(saved) // 3)]
         dev = saved[0].device if saved else gu.device
-        mask = _interior_mask(grid, dev)
-        g = []
-        for x in (gu, gv, gw):
-            g.append(torch.where(mask, x.to(torch.float32), 0.0) if x is not None
-                     else torch.zeros(grid.alloc_elems, dtype=torch.float32, device=dev))
-        # the adjoint writes every interior cell; the halo starts (and, as the
-        # periodic adjoint leaves it, stays) at zero, so the next call's
-        # incoming sensitivities have no stale values anywhere
-        g2 = [torch.zeros_like(t) for t in g]
+        # the incoming sensitivities of the interior, zeros elsewhere
+        g = _new_state(grid, dev)
+        h.keep_interior([None if x is None else x.to(torch.float32).contiguous() for x in (gu, gv, gw)], g)
+        # the adjoint writes every interior cell of its output, and neither reads
+        # nor keeps anything of its halo but the images it fills in itself
+        g2 = _new_state(grid, dev)
         for s in range(len(ckpts) - 1, -1, -1):
             n0 = s * every
             m = min(every, nsteps - n0)
@@ -85,8 +79,7 @@ class PWRollout(torch.autograd.Function):
                 h.adjoint(*q, *g, *g2, alpha=dt, flags=PW_ADJ_PERIODIC | PW_ADJ_ADD_LAMBDA)
                 g, g2 = g2, g
             del states
-        for t in g:
-            t.masked_fill_(~mask, 0.0)
+        h.keep_interior(g, g)
         return g[0], g[1], g[2], None, None, None, None
 
 

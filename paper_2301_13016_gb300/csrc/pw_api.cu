@@ -447,12 +447,17 @@ bool inject_failure(int kind) {
 cudaError_t set_smem_attr_once_impl(const void* kern, int bytes) {
     static std::mutex mu;
     static std::vector<std::pair<const void*, int>> done;   // (kernel, device)
+    static thread_local std::pair<const void*, int> last{nullptr, -1};   // this thread's last one found done
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    if (last.first == kern && last.second == dev) return cudaSuccess;
     std::lock_guard<std::mutex> lock(mu);
     for (auto& d : done)
-        if (d.first == kern && d.second == dev) return cudaSuccess;
+        if (d.first == kern && d.second == dev) {
+            last = d;
+            return cudaSuccess;
+        }
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     // all the shared memory an SM has, so that shared memory does not hold the
     // resident CTAs below what the registers allow (the kernels stage their
@@ -1163,6 +1168,29 @@ pw_status_t pw_fill_halo_periodic(pw_handle_t h, void* f, pw_stream_t stream) {
     cudaError_t e = launch_fill_halo(h->grid.dtype, to_dev(h->grid), &f, 1, h->num_sms,
                                      reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "halo fill launch");
+    return PW_OK;
+}
+
+pw_status_t pw_keep_interior(pw_handle_t h, const void* a, const void* b, const void* c, void* da, void* db, void* dc,
+                             int64_t n, pw_stream_t stream) {
+    PW_RANGE("pw_keep_interior");
+    if (!h) return fail(PW_ERR_ARG, "handle is NULL");
+    if (!da || !db || !dc) return fail(PW_ERR_ARG, "a field pointer is NULL");
+    if (n < alloc_elems_of(h->grid)) return fail(PW_ERR_ARG, "n is less than a field of this layout holds");
+    const void* src[3] = {a, b, c};
+    void* dst[3] = {da, db, dc};
+    if (da == db || da == dc || db == dc) return fail(PW_ERR_ARG, "outputs alias each other");
+    for (int q = 0; q < 3; ++q)
+        for (int d = 0; d < 3; ++d)
+            if (q != d && src[q] == dst[d]) return fail(PW_ERR_ARG, "an output aliases another field's input");
+    for (int q = 0; q < 3; ++q) {
+        const void* p[2] = {dst[q], src[q]};
+        pw_status_t st = check_device_ptrs(h, p, src[q] ? 2 : 1);
+        if (st != PW_OK) return st;
+    }
+    cudaError_t e = launch_keep_interior(h->grid.dtype, to_dev(h->grid), src, dst, (long long)n, h->num_sms,
+                                         reinterpret_cast<cudaStream_t>(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "interior copy launch");
     return PW_OK;
 }
 

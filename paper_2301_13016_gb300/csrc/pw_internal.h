@@ -198,6 +198,10 @@ int step_blocks_per_sm(pw_dtype_t dt, const TmaConfig& c);   // fused steps
 // Periodic images in the lateral halos of n fields (n <= 3), one launch.
 cudaError_t launch_fill_halo(pw_dtype_t dt, const GridDev& g, void* const* f, int n, int num_sms, cudaStream_t s);
 
+// dst = src on the interior, 0 in every other of the first n elements (three fields, one launch).
+cudaError_t launch_keep_interior(pw_dtype_t dt, const GridDev& g, const void* const* src, void* const* dst, long long n,
+                                 int num_sms, cudaStream_t s);
+
 // Bounded-wait self-test (see pw_selftest_wait_timeout).
 cudaError_t launch_selftest_wait(uint64_t limit_ns, int* err, cudaStream_t s);
 

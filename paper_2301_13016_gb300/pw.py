@@ -61,6 +61,7 @@ SIGNATURES = [
     ("pw_tendencies_host", ctypes.c_int, [_VP, _VP, _VP, _VP, _VP, _VP, _VP, _FP, _VP]),
     ("pw_tendencies_host_async", ctypes.c_int, [_VP, _VP, _VP, _VP, _VP, _VP, _VP, _FP, _VP]),
     ("pw_fill_halo_periodic", ctypes.c_int, [_VP, _VP, _VP]),
+    ("pw_keep_interior", ctypes.c_int, [_VP, _VP, _VP, _VP, _VP, _VP, _VP, ctypes.c_int64, _VP]),
     ("pw_adjoint", ctypes.c_int, [_VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP, _VP, ctypes.c_float, _I32, _VP]),
     ("pw_step", ctypes.c_int, [_VP, _VP, _VP, _VP, _VP, _VP, _VP, ctypes.c_float, _I32, _FP, _VP]),
     ("pw_step_to", ctypes.c_int, [_VP, _VP, _VP, _VP, _VP, _VP, _VP, ctypes.c_float, _FP, _VP]),
@@ -110,7 +111,7 @@ def lib():
 
 
 def _check(status, what):
-    if status != PW_OK:
+    if status:   # PW_OK is 0
         msg = lib().pw_last_error().decode(errors="replace")
         name = lib().pw_status_string(status).decode()
         raise PwError(status, f"{what}: {name}: {msg}")
@@ -126,10 +127,17 @@ def inject_failures(kind, count):
     _check(lib().pw_inject_failures(int(kind), int(count)), "pw_inject_failures")
 
 
+# the current stream's handle without building a torch.cuda.Stream (about 1 us
+# of the 13 us a tendencies() call of a small grid took)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream):
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 class Grid:
@@ -206,15 +214,18 @@ class Grid:
 def _ptr(t, grid, what, host=False):
     """Address of a field allocation: a CUDA tensor (a CPU one for the host
     entry point, host=True), of the grid's dtype, flat and large enough."""
+    # one test for a field that is fine (a 1-D tensor of more than one element
+    # is contiguous if and only if its stride is 1), then the reasons
+    if (isinstance(t, torch.Tensor) and t.is_cuda != host and t.dtype is grid.torch_dtype
+            and t.stride() == (1,) and t.numel() >= grid.alloc_elems):
+        return t.data_ptr()
     if not torch.is_tensor(t):
         raise TypeError(f"{what} must be a torch tensor")
     if host == t.is_cuda:
         raise ValueError(f"{what} must be a {'host' if host else 'CUDA'} tensor (got {t.device})")
     if t.dtype != grid.torch_dtype:
         raise TypeError(f"{what} has dtype {t.dtype}, grid stores {grid.torch_dtype}")
-    if t.dim() != 1 or not t.is_contiguous() or t.numel() < grid.alloc_elems:
-        raise ValueError(f"{what} must be a flat contiguous allocation of >= {grid.alloc_elems} elements")
-    return ctypes.c_void_p(t.data_ptr())
+    raise ValueError(f"{what} must be a flat contiguous allocation of >= {grid.alloc_elems} elements")
 
 
 def _scale_arg(scale):
@@ -359,6 +370,15 @@ class PW:
         _check(lib().pw_fill_halo_periodic(self.h, _ptr(f, self.grid, "f"), _stream_ptr(stream)),
                "pw_fill_halo_periodic")
 
+    def keep_interior(self, srcs, dsts, stream=None):
+        """dsts[q] = srcs[q] on the interior of levels 1..nz and 0 elsewhere, for
+        three fields in one launch (a source of None: zeros; its own output:
+        in place)."""
+        g = self.grid
+        n = min(t.numel() for t in dsts)
+        _check(lib().pw_keep_interior(self.h, *[None if t is None else _ptr(t, g, "src") for t in srcs],
+                                      *[_ptr(t, g, "dst") for t in dsts], n, _stream_ptr(stream)), "pw_keep_interior")
+
     def error_norms(self, test, ref, k0=1, k1=None, scale=1.0, stream=None):
         """(max|t-r|, max|r|, sum (t-r)^2, sum r^2) over levels k0..k1; ref is a
         dense (nz+2, ny+2, nx+2) float64 tensor (moved to the device)."""
@@ -478,7 +498,7 @@ class Batch:
         for name, lst in (("u", us), ("v", vs), ("w", ws), ("su", sus), ("sv", svs), ("sw", sws)):
             if len(lst) != n:
                 raise ValueError(f"{name}: need {n} tensors")
-            tabs.append((_VP * n)(*[_ptr(t, g, name).value for t, g in zip(lst, self.grids)]))
+            tabs.append((_VP * n)(*[_ptr(t, g, name) for t, g in zip(lst, self.grids)]))
         sp = _scale_arg(scale)
         _check(lib().pw_batch_tendencies(self.h, *tabs, sp[0] if sp else None, _stream_ptr(stream)),
                "pw_batch_tendencies")
