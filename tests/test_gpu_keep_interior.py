@@ -34,6 +34,19 @@ def test_keep_interior(n, in_place):
         assert torch.equal(a, b)
 
 
+def test_keep_interior_misaligned_buffers():
+    g = pwlib.Grid(30, 6, 4)
+    h = pwlib.PW(g, inputs.make_coeffs(4))
+    src = [torch.randn(g.alloc_elems + 1, device="cuda")[1:] for _ in range(3)]
+    dst = [g.alloc(fill=NAN) for _ in range(3)]
+    h.keep_interior(src, dst)
+    h.sync()
+    for s, d in zip(src, dst):
+        want = torch.zeros_like(d)
+        g.view(want)[1:-1, 1:-1, 1:-1] = g.view(s)[1:-1, 1:-1, 1:-1]
+        assert torch.equal(d, want)
+
+
 def test_keep_interior_refusals():
     g = pwlib.Grid(8, 4, 3)
     h = pwlib.PW(g, inputs.make_coeffs(3))
