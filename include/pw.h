@@ -129,7 +129,10 @@ pw_status_t pw_destroy(pw_handle_t h);
  * pw_adjoint: 0 = automatic (TMA k-march kernel when the layout and pointers
  * qualify, else the generic kernel; a width that is no multiple of 4 qualifies
  * for pw_tendencies and the step calls when no launch shape was fixed, nx >= 32
- * and the grid has at least 2^19 cells), 1 = generic kernel, 2 = TMA kernel,
+ * and the grid has at least 2^19 cells, FP32 steps wider than 80 columns on
+ * tiles that cover more than 1.1 x the width 2^21; a shape given to
+ * pw_set_tma_config, one read back by pw_get_tma_config among them, keeps such
+ * a width on the generic kernel), 1 = generic kernel, 2 = TMA kernel,
  * for widths that are a multiple of 4
  * (pw_tendencies and the step calls return PW_ERR_UNSUPPORTED/PW_ERR_ALIGN
  * when the layout or pointers do not qualify; pw_adjoint then runs the
@@ -152,7 +155,10 @@ pw_status_t pw_set_kernel(pw_handle_t h, int32_t kind);
  * multiple of 8, else (32, 4, 4, 4, 3)); (16, 4, 4, 4, 1) when nx <= 64; from
  * 2^18 cells up narrower tiles of as many cells, (16, 8, 4, 4, 1) and
  * (8, 16, 4, 4, 1) for FP32, (8, 16, 4, 8, 3), resp. (16, 8, 4, 4, 3), for 16
- * bits, where they are estimated to be faster (fewer cells beyond nx); nseg the
+ * bits, where they are estimated to be faster (fewer cells beyond nx); a width
+ * that is no multiple of 4 and at most 80 columns (16 bits: 96) packed rows: a
+ * CTA of 128 threads takes as many rows of ceil(nx/4) lanes x 4 cells as it has
+ * threads for (pw_get_tma_config reports these lanes and rows); nseg the
  * count estimated to fill the GPU best (segments of >= 2 levels; narrower tiles
  * and more segments only for a gain of 1.5 %).
  * Instantiated (lanes_x, ty, stages, cells, rows_per_thread): (32,4,4,4,1)

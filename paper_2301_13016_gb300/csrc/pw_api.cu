@@ -193,9 +193,13 @@ static pw_status_t encode_map_box(pw_handle_t h, const void* ptr, int box_w, int
     return PW_OK;
 }
 
-// Tensor map for the single-grid k-march shape (lx lanes x nc cells, ty rows).
-static pw_status_t encode_map(pw_handle_t h, const void* ptr, int lx, int ty, CUtensorMap* out, int nc = 4) {
-    return encode_map_box(h, ptr, tma_box_width(h->grid.dtype, lx, nc), ty + 2, out);
+// Tensor map for a launch shape of the single-grid k-march.
+static pw_status_t encode_map(pw_handle_t h, const void* ptr, const TmaConfig& c, CUtensorMap* out) {
+    if (c.rag == 2) {
+        const PackedRows p = packed_rows(h->grid.nx, (int)dtype_size(h->grid.dtype));
+        return encode_map_box(h, ptr, p.box_w, p.rows + 2, out);
+    }
+    return encode_map_box(h, ptr, tma_box_width(h->grid.dtype, c.lx, c.nc), c.ty + 2, out);
 }
 
 pw_status_t pw::encode_tensor_map(const pw_grid_t& g, const void* ptr, int lx, int ty, CUtensorMap* out, int nc,
@@ -298,6 +302,7 @@ static pw_status_t check_device_ptrs(pw_handle_t h, const void* const* ps, int n
 // as given, unset fields at the scalar defaults (32 lanes x 4 cells x 4 rows, 4
 // stages, one row per thread).  Otherwise 4 stages and one of these (lanes x
 // cells x rows), with the k segments, whichever march_cost puts lowest:
+//   narrow, no multiple of 4:   packed rows alone (kPackedNx);
 //   nx <= 64:                   16 x 4 x 4 alone;
 //   FP32:                       32 x 4 x 4, 16 x 4 x 8, 8 x 4 x 16;
 //   16-bit (source terms; steps when nx % 8 = 0):
@@ -314,6 +319,14 @@ static pw_status_t check_device_ptrs(pw_handle_t h, const void* const* ps, int n
 // keep the first shape: a call of that size is launch and latency.
 constexpr long long kShapeMinCells = 1 << 18;
 
+// Widths that are no multiple of 4 run in packed rows (PackedRows) up to these
+// columns.  Beyond, a row leaves threads idle (21 vectors: 126 of 128, 22: 110)
+// and the tiles fit better: FP32 source terms, packed / tiles, 69 x 787 x 89 32.3 /
+// 34.0 us, 79 x 203 x 69 9.9 / 9.9, 83 x 223 x 51 8.9 / 8.5; 16-bit ones and steps,
+// whose tiles are 64 columns wide, 83 x 223 x 51 8.8 / 9.5 and 11.7 / 14.5, 114 x 453
+// x 82 26.9 / 21.1 and 42.0 / 35.7.
+constexpr int kPackedNx = 80, kPackedNx16 = 96;
+
 // Estimated time of a march in units of one level of a full SM: `slots` CTAs
 // fit the GPU, each marches its levels after a start that costs as much as 1.6
 // of them (x pairs, whose levels take longer: 0.8); a last wave that leaves SMs
@@ -323,7 +336,8 @@ constexpr long long kShapeMinCells = 1 << 18;
 // choice is within 1 % (FP32 source terms), 2 % (16-bit), 3 to 4 % (steps) of
 // the sweep's best, where counting whole waves of (levels + 2) was 8 % off.
 static double march_cost(const pw_grid_t& gr, const TmaConfig& c, int n, int sms, int bps) {
-    const long long tiles = (long long)((gr.nx + c.nc * c.lx - 1) / (c.nc * c.lx)) * ((gr.ny + c.ty - 1) / c.ty);
+    const int rows = c.rag == 2 ? packed_rows(gr.nx, (int)dtype_size(gr.dtype)).rows : c.ty;
+    const long long tiles = (c.rag == 2 ? 1LL : (gr.nx + c.nc * c.lx - 1) / (c.nc * c.lx)) * ((gr.ny + rows - 1) / rows);
     const long long ctas = tiles * n, slots = (long long)sms * bps;
     const long long full = ctas / slots, rem = ctas - full * slots;
     const double w = c.xp ? 0.45 : 0.7;
@@ -349,7 +363,10 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
         if (u.stages) cand[0].stages = u.stages;
     } else {
         const bool half = dtype_size(gr.dtype) == 2, more = (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells;
-        if (gr.nx <= 64) {
+        const bool packed = gr.nx % 4 && gr.nx <= (half ? kPackedNx16 : kPackedNx);
+        if (packed) {
+            add(32, 4, 4, 0, 1);
+        } else if (gr.nx <= 64) {
             add(16, 4, 4, 0, 1);
         } else if (!half) {
             add(32, 4, 4, 0, 1);
@@ -362,7 +379,7 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
             add(32, 4, 4, 1, 1);
             if (more) add(16, 4, 8, 1, 1);
         }
-        for (int q = 0; q < nc; ++q) cand[q].rag = gr.nx % 4 != 0;
+        for (int q = 0; q < nc; ++q) cand[q].rag = gr.nx % 4 ? (packed ? 2 : 1) : 0;
     }
     TmaConfig best = cand[0];
     double lowest = 0.0;
@@ -386,20 +403,28 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
 // TMA k-march or generic kernel for the source terms and the steps: what
 // pw_set_kernel asked for, else TMA when the layout and every pointer qualify.
 // A width that is no multiple of 4 takes the k-march too (its RAG kernels) when
-// the shape is automatic and the grid has at least kRagMinCells cells:
-// measured on GB300, FP32 source terms, generic against k-march: 191x64x32
-// 5.7 / 6.0 us, 255x64x32 6.8 / 5.7, 63x256x64 11.3 / 8.2, 511x256x64 112 / 46,
-// 1021x1023x61 943 / 266.  A width below kRagMinNx would leave more than half
-// of the narrowest tile (64 columns) idle.  pw_set_kernel(2) refuses such a
-// width as it always has.
+// the shape is automatic and the grid has at least kRagMinCells cells; FP32
+// steps on tiles that cover more than 1.1 x the width (packed rows aside) from
+// kRagMinStepCells cells.  Measured on GB300, generic against k-march, us:
+//   source terms  FP32 41x168x69 (475 k cells) 6.6 / 7.0, 33x1000x16 6.8 / 6.6, 131x66x61 7.0 / 6.5, 229x57x47
+//                 7.8 / 7.2, 39x785x49 16.9 / 12.7, 511x256x64 111 / 44.5, 1021x1023x61 943 / 259; BF16 33x1000x16
+//                 7.0 / 6.8, 131x66x61 7.4 / 7.7, 511x64x17 7.2 / 6.8, 69x787x89 60.9 / 28.8;
+//   a step        FP32 33x129x125 (532 k) 8.2 / 9.2, 34x250x62 8.1 / 8.2, 65x129x64 8.0 / 7.9, 386x35x49 (662 k) 9.1 /
+//                 8.2, 39x785x49 20.7 / 17.0, 511x256x64 119 / 62; on tiles that fit badly 97x129x64 10.4 / 11.3,
+//                 102x489x17 10.5 / 13.2, 137x389x25 15.4 / 17.0, 135x129x128 (2.2 M) 25.7 / 24.4; BF16 33x1000x16
+//                 8.4 / 9.5, 97x129x64 11.3 / 11.1, 66x129x125 14.6 / 12.2, 39x785x49 19.3 / 16.8.
+// Below kRagMinNx columns the generic kernel stays: 9x2048x77 38.3 / 38.9, 17x2048x17 7.6 / 9.3, 13x1265x84 26.6 /
+// 21.3.  pw_set_kernel(2) refuses such a width as it always has.
 constexpr int kRagMinNx = 32;
-constexpr long long kRagMinCells = 1 << 19;
-static pw_status_t march_kernel_choice(pw_handle_t h, const void* const* bufs, int n, bool* use_tma, int* ox) {
+constexpr long long kRagMinCells = 1 << 19, kRagMinStepCells = 1 << 21;
+static pw_status_t march_kernel_choice(pw_handle_t h, bool step, const void* const* bufs, int n, bool* use_tma,
+                                       int* ox) {
     const char* why = "";
     const TmaConfig& u = h->tma_user;
     const pw_grid_t& gr = h->grid;
+    const bool loose = step && gr.dtype == PW_F32 && gr.nx > kPackedNx && 10LL * ((gr.nx + 31) / 32 * 32) > 11LL * gr.nx;
     const bool any_nx = h->kernel_kind == 0 && gr.nx >= kRagMinNx &&
-                        (long long)gr.nx * gr.ny * gr.nz >= kRagMinCells &&
+                        (long long)gr.nx * gr.ny * gr.nz >= (loose ? kRagMinStepCells : kRagMinCells) &&
                         !(u.lx || u.nc || u.ty || u.stages || u.rp);
     const bool layout_ok = tma_layout_ok(h->grid, ox, &why, any_nx);
     bool ptrs_ok = true;
@@ -703,9 +728,10 @@ pw_status_t pw_get_adjoint_config(pw_handle_t h, int32_t out[4]) {
 pw_status_t pw_get_tma_config(pw_handle_t h, int32_t step, int32_t out[6]) {
     if (!h || !out) return fail(PW_ERR_ARG, "handle or out is NULL");
     const TmaConfig c = choose_tma(h, step != 0);
-    out[0] = c.lx;
+    const PackedRows p = packed_rows(h->grid.nx, (int)dtype_size(h->grid.dtype));
+    out[0] = c.rag == 2 ? p.vec : c.lx;
     out[1] = c.nc;
-    out[2] = c.ty;
+    out[2] = c.rag == 2 ? p.rows : c.ty;
     out[3] = c.stages;
     out[4] = c.nseg;
     out[5] = c.xp ? 3 : c.rp;
@@ -743,13 +769,13 @@ pw_status_t pw_tendencies(pw_handle_t h, const void* u, const void* v, const voi
     int ox = 0;
     const void* all[6] = {u, v, w, su, sv, sw};
     bool use_tma = false;
-    pw_status_t kst = march_kernel_choice(h, all, 6, &use_tma, &ox);
+    pw_status_t kst = march_kernel_choice(h, false, all, 6, &use_tma, &ox);
     if (kst != PW_OK) return kst;
     if (use_tma) {
         TmaConfig c = choose_tma(h, false);
         CUtensorMap maps[3];
         for (int q = 0; q < 3; ++q) {
-            pw_status_t st = encode_map(h, ins[q], c.lx, c.ty, &maps[q], c.nc);
+            pw_status_t st = encode_map(h, ins[q], c, &maps[q]);
             if (st != PW_OK) return st;
         }
         cudaError_t e = launch_tend_tma(h->grid.dtype, g, ox, maps, su, sv, sw, sc, cf, h->d_err, c, s);
@@ -881,7 +907,7 @@ static pw_status_t tendencies_host(pw_handle_t h, const void* u, const void* v, 
     cfg.seg_count = 1;
     CUtensorMap maps[3];
     for (int q = 0; q < 3; ++q) {
-        pw_status_t st = encode_map(h, h->d_stage[q], cfg.lx, cfg.ty, &maps[q], cfg.nc);
+        pw_status_t st = encode_map(h, h->d_stage[q], cfg, &maps[q]);
         if (st != PW_OK) return st;
     }
     const GridDev gd = to_dev(g);
@@ -954,7 +980,7 @@ static pw_status_t step_pass(pw_handle_t h, const GridDev& g, const void* const*
     if (use_tma) {
         CUtensorMap maps[3];
         for (int q = 0; q < 3; ++q) {
-            pw_status_t st = encode_map(h, src[q], c.lx, c.ty, &maps[q], c.nc);
+            pw_status_t st = encode_map(h, src[q], c, &maps[q]);
             if (st != PW_OK) return st;
         }
         e = launch_step_tma(dtp, g, ox, maps, dst[0], dst[1], dst[2], sc, cf, dt, h->d_err, c, s);
@@ -987,7 +1013,7 @@ pw_status_t pw_step_to(pw_handle_t h, const void* u, const void* v, const void* 
     if (st != PW_OK) return st;
     bool use_tma = false;
     int ox = 0;
-    st = march_kernel_choice(h, bufs, 6, &use_tma, &ox);
+    st = march_kernel_choice(h, true, bufs, 6, &use_tma, &ox);
     if (st != PW_OK) return st;
     const GridDev g = to_dev(h->grid);
     CoefDev cf{h->tcx, h->tcy, h->d_tz};
@@ -1029,7 +1055,7 @@ pw_status_t pw_step(pw_handle_t h, void* u, void* v, void* w, void* tmp_u, void*
     }
     int ox = 0;
     bool use_tma = false;
-    sst = march_kernel_choice(h, bufs, 6, &use_tma, &ox);
+    sst = march_kernel_choice(h, true, bufs, 6, &use_tma, &ox);
     if (sst != PW_OK) return sst;
     // two steps per pass: TMA path, a lateral halo >= 2, and interior rows
     // starting at least 7 elements into their padded row (the q0 box begins

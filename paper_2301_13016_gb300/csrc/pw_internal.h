@@ -112,8 +112,25 @@ struct TmaConfig {
     int seg_count = 0;  // segments to launch (0 = all nseg)
     int rp = 1;         // rows per thread: 1, or 2 (packed FP32x2 arithmetic on row pairs)
     int xp = 0;         // 1: one row per thread, its nc cells packed as FP32x2 pairs (cell q, cell q + nc/2)
-    int rag = 0;        // 1: nx is no multiple of 4 (a row's last vector may hold 1 to nc cells)
+    int rag = 0;        // nx is no multiple of 4 (a row's last vector may hold 1 to nc cells): 1 tiles, 2 packed rows
 };
+
+// Packed rows (rag = 2): the 128 threads of a 32 x 4 CTA are dealt out to rows
+// of `vec` vectors of 4 cells, the whole width, as many rows as there are
+// threads and room in a 32 x 4 plane slot for; box_w: columns of the TMA box
+// (a multiple of 16 bytes).  Tiles of 32, 64 or 128 columns leave up to half
+// of their lanes beyond a narrow row's end: 33 x 1000 x 16 FP32 source terms 8.0
+// us on 64-column tiles, 6.7 packed, 6.8 on the generic kernel; 66 x 129 x 125 a
+// step 13.2 on 32-column tiles, 11.9 packed, 13.3 generic.
+struct PackedRows {
+    int vec, rows, box_w;
+};
+__host__ __device__ inline PackedRows packed_rows(int nx, int elem_size) {
+    const int padx = 16 / elem_size, vec = (nx + 3) / 4;
+    const int box_w = (4 * vec + padx - 1) / padx * padx + 2 * padx;
+    const int fit = 6 * (128 + 2 * padx) / box_w - 2, rows = 128 / vec;
+    return PackedRows{vec, rows < fit ? rows : fit, box_w};
+}
 
 // Launch shape of the two-step (temporal blocking) k-march kernel.
 struct Step2Config {
