@@ -318,6 +318,7 @@ static pw_status_t check_device_ptrs(pw_handle_t h, const void* const* ps, int n
 // 122 -> 115, 512x512x64 (segments alone) 61 -> 55.  Grids below kShapeMinCells
 // keep the first shape: a call of that size is launch and latency.
 constexpr long long kShapeMinCells = 1 << 18;
+constexpr int kMaxGridY = 65535;   // CTAs of a launch along y (and z)
 
 // Widths that are no multiple of 4 run in packed rows (PackedRows) up to these
 // columns.  Beyond, a row leaves threads idle (21 vectors: 126 of 128, 22: 110)
@@ -423,7 +424,9 @@ static pw_status_t march_kernel_choice(pw_handle_t h, bool step, const void* con
     const TmaConfig& u = h->tma_user;
     const pw_grid_t& gr = h->grid;
     const bool loose = step && gr.dtype == PW_F32 && gr.nx > kPackedNx && 10LL * ((gr.nx + 31) / 32 * 32) > 11LL * gr.nx;
-    const bool any_nx = h->kernel_kind == 0 && gr.nx >= kRagMinNx &&
+    const bool packed = gr.nx <= (gr.dtype == PW_F32 ? kPackedNx : kPackedNx16);
+    const int rows = packed ? packed_rows(gr.nx, (int)dtype_size(gr.dtype)).rows : 4;   // the lowest tile's
+    const bool any_nx = h->kernel_kind == 0 && gr.nx >= kRagMinNx && gr.ny <= (long long)kMaxGridY * rows &&
                         (long long)gr.nx * gr.ny * gr.nz >= (loose ? kRagMinStepCells : kRagMinCells) &&
                         !(u.lx || u.nc || u.ty || u.stages || u.rp);
     const bool layout_ok = tma_layout_ok(h->grid, ox, &why, any_nx);
@@ -1148,7 +1151,9 @@ pw_status_t pw_adjoint(pw_handle_t h, const void* u, const void* v, const void* 
     const AdjMode mode = !(flags & PW_ADJ_PERIODIC) ? ADJ_OPEN : (gr.nx % 4 == 0 ? ADJ_PERIODIC : ADJ_PERIODIC_ANY);
     const bool size_ok = mode != ADJ_PERIODIC_ANY || (h->kernel_kind == 0 && gr.nx >= kRagMinNx && gr.ny >= 8 &&
                                                       (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells);
-    if (h->kernel_kind != 1 && ptrs_ok && size_ok && (mode == ADJ_PERIODIC || !fixed) &&
+    // the full array and odd widths were the gather kernel's, which takes any height and depth
+    const bool fits = mode == ADJ_PERIODIC || (gr.ny + 2LL <= 8LL * kMaxGridY && gr.nz <= 64LL * kMaxGridY);
+    if (h->kernel_kind != 1 && ptrs_ok && size_ok && fits && (mode == ADJ_PERIODIC || !fixed) &&
         tma_layout_ok(gr, &ox, &why, mode != ADJ_PERIODIC)) {
         const GridDev g = to_dev(gr);
         if (mode == ADJ_PERIODIC) {   // the sensitivities need periodic halos too
