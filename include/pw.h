@@ -313,7 +313,7 @@ pw_status_t pw_step_to(pw_handle_t h, const void *u, const void *v, const void *
  * in periodic mode for widths that are a multiple of 4, the lateral halos of
  * lsu, lsv, lsw being first overwritten with their periodic images (their halo
  * values carry no meaning in this mode); unless pw_set_adjoint_config fixed a
- * shape, in periodic mode for other widths (from 32 columns and 2^18 cells up;
+ * shape other than (4, 8, 3), in periodic mode for other widths (from 32 columns and 2^18 cells up;
  * the halos of lsu, lsv, lsw are neither read nor written then) and without
  * PW_ADJ_PERIODIC for any width.  Otherwise the generic gather kernel runs.  A
  * term whose sensitivity is exactly 0 is skipped, but for the periodic k-march
@@ -326,18 +326,21 @@ pw_status_t pw_adjoint(pw_handle_t h, const void *u, const void *v, const void *
                        void *gu, void *gv, void *gw, float alpha, int32_t flags, pw_stream_t stream);
 
 /*
- * Launch shape of the periodic TMA adjoint on this handle (0 = automatic,
+ * Launch shape of the TMA adjoint on this handle (0 = automatic,
  * field by field): cells = consecutive cells a thread owns along x, ty = rows
  * per CTA, stages = ring slots of the six planes (levels k, k+1 resident, the
  * rest in flight), nseg = CTAs along z (1..nz; automatic: the count estimated
  * to fill the GPU best, segments of >= 4 levels; a segment never exceeds 126
- * levels).  Instantiated (cells, ty, stages): (4,5,4) (4,4,4) (4,6,4) (2,4,4)
+ * levels, 64 where zero sensitivities are skipped, so nseg is raised to that).
+ * Instantiated (cells, ty, stages): (4,5,4) (4,4,4) (4,6,4) (2,4,4)
  * (2,5,4) (2,6,4) (2,8,4) (2,8,3), a CTA covering 32*cells columns with one
- * warp per row; others give PW_ERR_UNSUPPORTED, a negative value or nseg > nz
- * PW_ERR_ARG.  Automatic: (4,6,4), and from 2^18 cells up 4 cells x 8 rows with
- * 3 slots and 64 columns a CTA.  Each cell's arithmetic is the same in every
+ * warp per row, and (4,8,3), 64 columns with two rows per warp; others give
+ * PW_ERR_UNSUPPORTED, a negative value or nseg > nz PW_ERR_ARG.  Automatic:
+ * (4,6,4) for periodic grids below 2^18 cells and widths that are a multiple of
+ * 4, else (4,8,3).  The modes that skip zero sensitivities have (4,8,3) alone; nseg
+ * by itself fixes no shape.  Each cell's arithmetic is the same in every
  * shape.  pw_get_adjoint_config: out = {cells, ty, stages, nseg} that the next
- * periodic TMA adjoint call will use.
+ * periodic TMA adjoint call will use; pw_set_adjoint_config takes it back.
  */
 pw_status_t pw_set_adjoint_config(pw_handle_t h, int32_t cells, int32_t ty, int32_t stages, int32_t nseg);
 pw_status_t pw_get_adjoint_config(pw_handle_t h, int32_t out[4]);

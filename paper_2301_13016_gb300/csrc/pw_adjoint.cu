@@ -249,11 +249,10 @@ struct AdjLayout {
     static constexpr uint32_t TX_BYTES = 6u * FIELD_RAW * 4u;
     // the ring, one mbarrier per slot, 4 flag words, then the vertical
     // coefficients {tzc1, tzc2, tzd1, tzd2} of levels kb-1..ke+1 of the CTA's k
-    // segment, one float4 per level (the host keeps a segment within MAX_SEG
-    // levels; CHECKED within MAX_SEG_CHECKED, the bits of its mask of levels to redo)
-    static constexpr int MAX_SEG = 126, MAX_SEG_CHECKED = 64;
+    // segment, one float4 per level (the host keeps a segment within kAdjMaxSeg
+    // levels; CHECKED within kAdjMaxSegChecked)
     static constexpr size_t CTZ_OFF = (((size_t)S * STAGE * 4 + S * sizeof(uint64_t) + 16 + 15) / 16) * 16;
-    static constexpr size_t SMEM = CTZ_OFF + (size_t)(MAX_SEG + 2) * sizeof(float4);
+    static constexpr size_t SMEM = CTZ_OFF + (size_t)(kAdjMaxSeg + 2) * sizeof(float4);
 };
 
 struct AdjMaps {
@@ -661,9 +660,17 @@ __global__ void __launch_bounds__((AdjLayout<NA, LX, TY, S>::THREADS), (adj_min_
 #define PW_ADJ_CONFIGS(X) X(4, 5, 4) X(4, 4, 4) X(4, 6, 4) X(2, 4, 4) X(2, 5, 4) X(2, 6, 4) X(2, 8, 4) X(2, 8, 3)
 #define PW_ADJ_AUTO(X) X(4, 16, 8, 3)
 
-AdjConfig adjoint_default_config() { return AdjConfig{4, 6, 4, 0}; }
+AdjConfig adjoint_shape(const AdjConfig& u) {
+    AdjConfig c{u.na ? u.na : 4, u.ty ? u.ty : 6, u.stages ? u.stages : 4, u.nseg, 32};
+    if (c.na == 4 && c.ty == 8 && c.stages == 3) c.lx = 16;
+    return c;
+}
 
 bool adjoint_config_supported(const AdjConfig& c) {
+#define PW_AB(NA_, LX_, TY_, S_) \
+    if (c.lx == LX_ && c.na == NA_ && c.ty == TY_ && c.stages == S_) return true;
+    PW_ADJ_AUTO(PW_AB)
+#undef PW_AB
 #define PW_AS(NA_, TY_, S_) \
     if (c.lx == 32 && c.na == NA_ && c.ty == TY_ && c.stages == S_) return true;
     PW_ADJ_CONFIGS(PW_AS)
@@ -679,7 +686,7 @@ static cudaError_t adj_inst(const AdjConfig& c, int* bps, const GridDev& g, cons
     cudaError_t e = set_smem_attr_once(kern, (int)L::SMEM);
     if (e != cudaSuccess) return e;
     if (bps) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, kern, L::THREADS, L::SMEM);
-    constexpr int most = CHECKED ? L::MAX_SEG_CHECKED : L::MAX_SEG;
+    constexpr int most = CHECKED ? kAdjMaxSegChecked : kAdjMaxSeg;
     const int nseg = std::max(c.nseg, (g.nz + most - 1) / most);
     const int wx = ge.ihi - ge.i0 + 1, wy = ge.jhi - ge.j0 + 1;
     dim3 grid((wx + L::TX - 1) / L::TX, (wy + TY - 1) / TY, nseg);

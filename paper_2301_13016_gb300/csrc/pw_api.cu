@@ -668,6 +668,13 @@ static Step2Config choose_step2(pw_handle_t h) {
     return c;
 }
 
+// The caller fixed a shape that only the periodic mode of widths that are a
+// multiple of 4 is instantiated for.
+static bool adj_fixed(pw_handle_t h) {
+    const AdjConfig& u = h->adj_user;
+    return (u.na || u.ty || u.stages) && adjoint_shape(u).lx != 16;
+}
+
 // Launch shape of the TMA adjoint (periodic or open mode): each field the user
 // fixed, else 32 lanes x 4 cells x 6 rows with 4 slots for periodic grids below
 // kShapeMinCells, and 16 lanes x 4 cells x 8 rows with 3 slots otherwise; k
@@ -677,15 +684,14 @@ static Step2Config choose_step2(pw_handle_t h) {
 static AdjConfig choose_adjoint(pw_handle_t h, AdjMode mode) {
     AdjConfig& cache = h->adj_auto[mode];
     if (cache.na) return cache;
-    const AdjConfig d = adjoint_default_config();
     const AdjConfig& u = h->adj_user;
     const pw_grid_t& gr = h->grid;
-    AdjConfig c{u.na ? u.na : d.na, u.ty ? u.ty : d.ty, u.stages ? u.stages : d.stages, u.nseg, 32};
+    AdjConfig c = adjoint_shape(u);
     if (mode != ADJ_PERIODIC || (!u.na && !u.ty && !u.stages && (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells))
         c = AdjConfig{4, 8, 3, u.nseg, 16};
     if (!c.nseg) {
         const AdjGeom ge = adj_geom(gr, 0, mode);
-        const int wx = ge.ihi - ge.i0 + 1, wy = ge.jhi - ge.j0 + 1, tx = c.lx * c.na;
+        const int wx = std::max(1, ge.ihi - ge.i0 + 1), wy = std::max(1, ge.jhi - ge.j0 + 1), tx = c.lx * c.na;
         const long long tiles = (long long)((wx + tx - 1) / tx) * ((wy + c.ty - 1) / c.ty);
         const int bps = std::max(1, adjoint_blocks_per_sm(c, mode != ADJ_PERIODIC));
         const long long slots = (long long)h->num_sms * bps;
@@ -699,7 +705,8 @@ static AdjConfig choose_adjoint(pw_handle_t h, AdjMode mode) {
             c.nseg = n;
         }
     }
-    if (c.nseg > gr.nz) c.nseg = gr.nz;
+    const int most = mode == ADJ_PERIODIC ? kAdjMaxSeg : kAdjMaxSegChecked;
+    c.nseg = std::min(std::max(c.nseg, (gr.nz + most - 1) / most), (int)gr.nz);
     cache = c;
     return c;
 }
@@ -708,19 +715,18 @@ pw_status_t pw_set_adjoint_config(pw_handle_t h, int32_t cells, int32_t ty, int3
     if (!h) return fail(PW_ERR_ARG, "handle is NULL");
     if (cells < 0 || ty < 0 || stages < 0) return fail(PW_ERR_ARG, "cells, ty and stages must be >= 0");
     if (nseg < 0 || nseg > h->grid.nz) return fail(PW_ERR_ARG, "nseg must be in 0..nz");
-    const AdjConfig d = adjoint_default_config();
-    const AdjConfig c{cells ? cells : d.na, ty ? ty : d.ty, stages ? stages : d.stages, nseg, 32};
+    const AdjConfig c = adjoint_shape(AdjConfig{cells, ty, stages, nseg});
     if (!adjoint_config_supported(c))
         return fail(PW_ERR_UNSUPPORTED, "no TMA adjoint instance for cells=%d ty=%d stages=%d", c.na, c.ty,
                     c.stages);
     h->adj_user = AdjConfig{cells, ty, stages, nseg};
-    for (auto& c : h->adj_auto) c = AdjConfig{};
+    for (auto& a : h->adj_auto) a = AdjConfig{};
     return PW_OK;
 }
 
 pw_status_t pw_get_adjoint_config(pw_handle_t h, int32_t out[4]) {
     if (!h || !out) return fail(PW_ERR_ARG, "handle or out is NULL");
-    const AdjConfig c = choose_adjoint(h, ADJ_PERIODIC);
+    const AdjConfig c = choose_adjoint(h, h->grid.nx % 4 && !adj_fixed(h) ? ADJ_PERIODIC_ANY : ADJ_PERIODIC);
     out[0] = c.na;
     out[1] = c.ty;
     out[2] = c.stages;
@@ -1146,14 +1152,12 @@ pw_status_t pw_adjoint(pw_handle_t h, const void* u, const void* v, const void* 
     // kShapeMinCells cells up (the ring of cells gathered by a second launch is
     // then a small part), both with the automatic shape.
     const pw_grid_t& gr = h->grid;
-    const AdjConfig& au = h->adj_user;
-    const bool fixed = au.na || au.ty || au.stages || au.nseg;
     const AdjMode mode = !(flags & PW_ADJ_PERIODIC) ? ADJ_OPEN : (gr.nx % 4 == 0 ? ADJ_PERIODIC : ADJ_PERIODIC_ANY);
     const bool size_ok = mode != ADJ_PERIODIC_ANY || (h->kernel_kind == 0 && gr.nx >= kRagMinNx && gr.ny >= 8 &&
                                                       (long long)gr.nx * gr.ny * gr.nz >= kShapeMinCells);
     // the full array and odd widths were the gather kernel's, which takes any height and depth
     const bool fits = mode == ADJ_PERIODIC || (gr.ny + 2LL <= 8LL * kMaxGridY && gr.nz <= 64LL * kMaxGridY);
-    if (h->kernel_kind != 1 && ptrs_ok && size_ok && fits && (mode == ADJ_PERIODIC || !fixed) &&
+    if (h->kernel_kind != 1 && ptrs_ok && size_ok && fits && (mode == ADJ_PERIODIC || !adj_fixed(h)) &&
         tma_layout_ok(gr, &ox, &why, mode != ADJ_PERIODIC)) {
         const GridDev g = to_dev(gr);
         if (mode == ADJ_PERIODIC) {   // the sensitivities need periodic halos too

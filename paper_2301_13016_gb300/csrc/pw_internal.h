@@ -205,7 +205,12 @@ cudaError_t launch_adjoint_tma(const GridDev& g, const AdjGeom& ge, AdjMode mode
                                const float* const* q6, float* const* g3, float alpha, int accumulate, int add_lambda,
                                const CoefDev& cf, int* err, const AdjConfig& c, int num_sms, cudaStream_t s);
 bool adjoint_config_supported(const AdjConfig& c);
-AdjConfig adjoint_default_config();
+// The shape of which a caller gave some fields (0: the default's); (4, 8, 3),
+// the automatic one of larger grids, has 16 lanes per row, the others 32.
+AdjConfig adjoint_shape(const AdjConfig& u);
+// Levels a k segment may have: the kernel's coefficient table, and (every mode
+// but ADJ_PERIODIC) the bits of its mask of levels to redo.
+constexpr int kAdjMaxSeg = 126, kAdjMaxSegChecked = 64;
 int adjoint_blocks_per_sm(const AdjConfig& c, bool checked);   // checked: every mode but ADJ_PERIODIC
 
 // Blocks of the TMA kernel resident per SM for a config (0 if it cannot launch).
