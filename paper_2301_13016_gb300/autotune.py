@@ -22,8 +22,9 @@ BATCH_CANDIDATES = [dict(lanes_x=lx, ty=ty, stages=4, ctas_per_sm=c, rows=rp, ce
                                            (16, 8, 4, 2), (32, 8, 4, 3), (16, 8, 4, 3), (16, 8, 8, 3), (16, 4, 8, 3),
                                            (8, 8, 8, 3), (8, 16, 8, 3), (8, 16, 4, 1), (32, 16, 4, 1))
                     for c in (0, 2)]
+AUTOMATIC = dict(lanes_x=0, ty=0, stages=0, nseg=0, cells=0, rows=0)   # the library's own choice
 GRID_CANDIDATES = [dict(lanes_x=lx, ty=ty, stages=st, nseg=ns, cells=nc, rows=rp)
-                   for lx, ty, st, nc, rp in ((32, 4, 4, 4, 1), (32, 8, 4, 4, 1), (32, 8, 6, 4, 1), (16, 4, 4, 4, 1),
+                   for lx, ty, st, nc, rp in ((0, 0, 0, 0, 0), (32, 4, 4, 4, 1), (32, 8, 4, 4, 1), (32, 8, 6, 4, 1), (16, 4, 4, 4, 1),
                                               (16, 8, 4, 4, 1), (16, 4, 4, 8, 1), (16, 8, 4, 8, 1), (32, 8, 4, 4, 2),
                                               (32, 16, 4, 4, 2), (16, 8, 4, 4, 2), (16, 4, 4, 8, 3),
                                               (16, 8, 4, 8, 3), (16, 16, 4, 8, 3), (32, 4, 4, 4, 3), (32, 8, 4, 4, 3),
@@ -107,20 +108,39 @@ def tune_batch(batch, fields, candidates=None, warmup=2, reps=5, cache_path=None
     return best, times
 
 
+def _kernel(handle, fields, config):
+    """The kernel (PW.last_kernel) that tendencies() takes with this shape; None
+    if the shape is refused."""
+    try:
+        handle.set_tma_config(**config)
+    except RuntimeError:
+        return None
+    handle.tendencies(*fields)
+    return handle.last_kernel
+
+
 def tune_grid(handle, fields, candidates=None, warmup=2, reps=5, cache_path=None, force=False):
     """Pick and apply the fastest single-grid k-march shape for `handle`.
-    fields = (u, v, w, su, sv, sw) flat device tensors.  Returns (config, times)."""
+    fields = (u, v, w, su, sv, sw) flat device tensors.  Returns (config, times).
+
+    A width that is no multiple of 4 runs on the k-march with the automatic
+    shape only: there, a candidate or cached shape that takes another kernel
+    than the automatic one is left out."""
     cache_path = cache_path or _default_cache()
     g = handle.grid
     key = _signature("grid", [[g.nx, g.ny, g.nz]], g.dtype)
+    auto = _kernel(handle, fields, AUTOMATIC) if g.nx % 4 else None
     cached = _load(cache_path).get(key)
-    if cached and not force:
+    if cached and not force and (auto is None or _kernel(handle, fields, cached["config"]) == auto):
         handle.set_tma_config(**cached["config"])
         return cached["config"], cached.get("times", {})
+    candidates = candidates or GRID_CANDIDATES
+    if auto is not None:
+        candidates = [c for c in candidates if _kernel(handle, fields, c) == auto] or [AUTOMATIC]
     stream = torch.cuda.current_stream()
     times = {}
     best, best_ms = None, float("inf")
-    for c in candidates or GRID_CANDIDATES:
+    for c in candidates:
         if c["nseg"] > g.nz // 2:
             continue
         try:
