@@ -381,6 +381,9 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
             if (more) add(16, 4, 8, 1, 1);
         }
         for (int q = 0; q < nc; ++q) cand[q].rag = gr.nx % 4 ? (packed ? 2 : 1) : 0;
+        const long long cells = (long long)gr.nx * gr.ny * gr.nz;   // (see tma_min_blocks)
+        if (step && gr.nx % 4 == 0 && !cand[0].xp)
+            cand[0].few = gr.nx > 64 ? cells <= (1 << 20) : gr.nx < 64 && cells < (1 << 17);
     }
     TmaConfig best = cand[0];
     double lowest = 0.0;

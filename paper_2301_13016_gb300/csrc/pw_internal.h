@@ -113,6 +113,7 @@ struct TmaConfig {
     int rp = 1;         // rows per thread: 1, or 2 (packed FP32x2 arithmetic on row pairs)
     int xp = 0;         // 1: one row per thread, its nc cells packed as FP32x2 pairs (cell q, cell q + nc/2)
     int rag = 0;        // nx is no multiple of 4 (a row's last vector may hold 1 to nc cells): 1 tiles, 2 packed rows
+    int few = 0;        // 1: the scalar step's instance for few cells (see tma_min_blocks)
 };
 
 // Packed rows (rag = 2): the 128 threads of a 32 x 4 CTA are dealt out to rows

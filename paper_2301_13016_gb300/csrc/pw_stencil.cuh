@@ -915,9 +915,17 @@ struct TmaLayout {
 // BF16 against the compiler's 210 registers, as more CTAs per SM hide more
 // latency; 128 spills and 200 leaves 2 CTAs per SM, both slower).
 //
-// The scalar steps' cap (PW_STEP_REGS) is for FP32 storage: 16-bit ones, at most 64
-// columns wide, take 4.74 us at 64^3 without it and 4.95 with it, 32 x 69 x 25 5.37 and 5.58.
-template <typename T, int LX, int TY, int S, int NC = 4, int RP = 1, int XP = 0, int MODE = MODE_TEND, int RAG = 0>
+// FEW: the scalar step of a grid of few cells, which waits for a level's latency
+// and has no use for a fifth CTA per SM: the compiler's registers on 32 lanes,
+// one test for the images (store_field) on 16.  us a step, capped at PW_STEP_REGS
+// with single predicated stores / FEW: 120 x 64 x
+// 17 5.2 / 4.8, 88 x 18 x 43 5.3 / 4.9, 128 x 128 x 64 8.4 / 8.2 (256 x 128 x 64 13.2 /
+// 13.5: not above 2^20 cells); 32 x 69 x 25 5.1 / 4.9, 52 x 52 x 43 4.9 / 4.8 (44 x 119
+// x 33 5.2 / 5.5, 64 columns 0.1 slower: not from 2^17 cells, not at 64 columns).
+// The cap is for FP32 storage: 16-bit scalar steps, at most 64 columns wide, take
+// 4.74 us at 64^3 without it and 4.95 with it, 32 x 69 x 25 5.37 and 5.58.
+template <typename T, int LX, int TY, int S, int NC = 4, int RP = 1, int XP = 0, int MODE = MODE_TEND, int RAG = 0,
+          int FEW = 0>
 constexpr int tma_min_blocks() {
     using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
     constexpr int by_smem = (int)((227u * 1024u) / (L::SMEM + 1024u));   // 1 KB per CTA is the system's
@@ -926,7 +934,7 @@ constexpr int tma_min_blocks() {
         (L::PD_SMEM && NC == 8)
             ? 65536 / (L::THREADS * PW_TMA_REGS_XP)
             : (NC * RP == 8 ? 65536 / (L::THREADS * PW_TMA_REGS8)
-                            : (MODE == MODE_STEP && !L::PACKED && !RAG && sizeof(T) == 4
+                            : (MODE == MODE_STEP && !L::PACKED && !RAG && !FEW && sizeof(T) == 4
                                    ? 65536 / (L::THREADS * PW_STEP_REGS)
                                    : PW_TMA_MAX_MINB));
     constexpr int m0 = by_smem < by_threads ? by_smem : by_threads;
@@ -1042,7 +1050,7 @@ __device__ __forceinline__ void load_pairs_sa(uint32_t a, float2 (&o)[NC / 2]) {
 // of the padded row or the tensor map's zero fill, and not stored.
 // RAG = 2: the same with packed rows (`prows` of them, see PackedRows), one tile
 // column; every x neighbour comes from the staged row, as rows end inside warps.
-template <typename T, int LX, int TY, int S, int MODE, int NC = 4, int RP = 1, int XP = 0, int RAG = 0>
+template <typename T, int LX, int TY, int S, int MODE, int NC = 4, int RP = 1, int XP = 0, int RAG = 0, int FEW = 0>
 __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP, XP>& sm, const CUtensorMap* tm_u,
                                            const CUtensorMap* tm_v, const CUtensorMap* tm_w, T* __restrict__ o0,
                                            T* __restrict__ o1, T* __restrict__ o2, const GridDev& g, const int ox,
@@ -1127,7 +1135,6 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
     const long long row_off = g.origin + (long long)j * g.pj + i0;
     // the arithmetic runs on stored values, the storage scales folded into the
     // coefficients kc
-    const int nzp2 = nz + 2;
     const unsigned FULL = 0xffffffffu;
     auto ld = [&](const T* p, float (&o)[NC]) { loadv<NC>(p, o); };
     auto ld1 = [&](const T* p) { return Store<T>::to_f(*p); };
@@ -1248,7 +1255,7 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
                             return;
                         }
                     }
-                    Epilogue<T, MODE>::template store_field<NC, (XP != 0)>(of, o, a, g, j + half, i0, err);
+                    Epilogue<T, MODE>::template store_field<NC, (XP != 0 || (FEW && LX == 16))>(of, o, a, g, j + half, i0, err);
                 };
                 if (valid) field_row(0);
                 if (RP == 2 && valid2) field_row(1);
@@ -1386,9 +1393,9 @@ __device__ __forceinline__ bool march_tile(const MarchSmem<T, LX, TY, S, NC, RP,
 }
 
 // One grid, one tile per CTA: blockIdx = (tile column, tile row, k segment).
-template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP, int RAG>
+template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP, int RAG, int FEW>
 __global__ void __launch_bounds__(TmaLayout<T, LX, TY, S, NC, RP, XP>::THREADS,
-                                  (tma_min_blocks<T, LX, TY, S, NC, RP, XP, MODE, RAG>()))
+                                  (tma_min_blocks<T, LX, TY, S, NC, RP, XP, MODE, RAG, FEW>()))
     tma_kernel(const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_v,
                const __grid_constant__ CUtensorMap tm_w, T* __restrict__ o0, T* __restrict__ o1,
                T* __restrict__ o2, const GridDev g, const int ox, const int nseg, const int seg0, const FoldedCoef kc,
@@ -1400,8 +1407,8 @@ __global__ void __launch_bounds__(TmaLayout<T, LX, TY, S, NC, RP, XP>::THREADS,
     const int ke = (int)(((long long)(bz + 1) * g.nz) / nseg);
     if (ke < kb) return;   // empty k segment (the host never launches one)
     uint32_t ring = 0;
-    march_tile<T, LX, TY, S, MODE, NC, RP, XP, RAG>(sm, &tm_u, &tm_v, &tm_w, o0, o1, o2, g, ox, kc, dt, blockIdx.x,
-                                               blockIdx.y, kb, ke, ring, err, true, prows);
+    march_tile<T, LX, TY, S, MODE, NC, RP, XP, RAG, FEW>(sm, &tm_u, &tm_v, &tm_w, o0, o1, o2, g, ox, kc, dt, blockIdx.x,
+                                                    blockIdx.y, kb, ke, ring, err, true, prows);
 }
 
 // Instantiated single-grid launch shapes: (lanes per row, rows, stages, cells
@@ -1432,7 +1439,7 @@ constexpr bool rag_ok() {
 template <typename T, int NC, int RP, int XP = 0>
 constexpr bool nc_ok() { return (NC == 4 && RP == 1 && XP == 0) || sizeof(T) == 2; }
 
-template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP, int RAG = 0>
+template <typename T, int LX, int TY, int S, int MODE, int NC, int RP, int XP, int RAG = 0, int FEW = 0>
 static cudaError_t launch_tma_inst(const GridDev& g, int ox, const CUtensorMap* maps, void* o0, void* o1,
                                    void* o2, const Scales& sc, const CoefDev& cf, float dt, int* err, int nseg,
                                    int seg0, int seg_count, cudaStream_t s) {
@@ -1440,7 +1447,7 @@ static cudaError_t launch_tma_inst(const GridDev& g, int ox, const CUtensorMap* 
     return cudaErrorInvalidConfiguration;
   } else {
     using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
-    auto kern = tma_kernel<T, LX, TY, S, MODE, NC, RP, XP, RAG>;
+    auto kern = tma_kernel<T, LX, TY, S, MODE, NC, RP, XP, RAG, FEW>;
     cudaError_t e = set_smem_attr_once(kern, (int)L::SMEM);
     if (e != cudaSuccess) return e;
     if (seg_count <= 0) seg_count = nseg - seg0;
@@ -1461,6 +1468,14 @@ static cudaError_t launch_tma_mode(const GridDev& g, int ox, const CUtensorMap* 
     if (c.lx == LX_ && c.ty == TY_ && c.stages == S_ && c.nc == NC_ && c.rp == RP_ && c.xp == XP_)      \
         return launch_tma_inst<T, LX_, TY_, S_, MODE, NC_, RP_, XP_>(g, ox, maps, o0, o1, o2, sc, cf, dt, err, \
                                                                      c.nseg, c.seg0, c.seg_count, s);
+    if constexpr (MODE == MODE_STEP) {
+        if (c.few && c.lx == 32)
+            return launch_tma_inst<T, 32, 4, 4, MODE, 4, 1, 0, 0, 1>(g, ox, maps, o0, o1, o2, sc, cf, dt, err, c.nseg,
+                                                                     c.seg0, c.seg_count, s);
+        if (c.few)
+            return launch_tma_inst<T, 16, 4, 4, MODE, 4, 1, 0, 0, 1>(g, ox, maps, o0, o1, o2, sc, cf, dt, err, c.nseg,
+                                                                     c.seg0, c.seg_count, s);
+    }
     if (c.rag == 2)
         return launch_tma_inst<T, 32, 4, 4, MODE, 4, 1, 0, 2>(g, ox, maps, o0, o1, o2, sc, cf, dt, err, c.nseg, c.seg0,
                                                               c.seg_count, s);
@@ -1478,11 +1493,11 @@ static cudaError_t launch_tma_mode(const GridDev& g, int ox, const CUtensorMap* 
     return cudaErrorInvalidConfiguration;
 }
 
-template <typename T, int MODE, int RAG, int LX, int TY, int S, int NC, int RP, int XP>
+template <typename T, int MODE, int RAG, int LX, int TY, int S, int NC, int RP, int XP, int FEW = 0>
 static int blocks_inst() {
     int n = 0;
     if constexpr (nc_ok<T, NC, RP, XP>() && (RAG != 1 || rag_ok<T, MODE, NC, XP>())) {
-        auto kern = tma_kernel<T, LX, TY, S, MODE, NC, RP, XP, RAG>;
+        auto kern = tma_kernel<T, LX, TY, S, MODE, NC, RP, XP, RAG, FEW>;
         using L = TmaLayout<T, LX, TY, S, NC, RP, XP>;
         if (set_smem_attr_once(kern, (int)L::SMEM) != cudaSuccess) return 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, L::THREADS, L::SMEM) != cudaSuccess) return 0;
@@ -1496,6 +1511,10 @@ static int blocks_per_sm_mode(const TmaConfig& c) {
 #define PW_OCC(LX_, TY_, S_, NC_, RP_, XP_)                                                            \
     if (c.lx == LX_ && c.ty == TY_ && c.stages == S_ && c.nc == NC_ && c.rp == RP_ && c.xp == XP_)     \
         return blocks_inst<T, MODE, PW_OCC_RAG, LX_, TY_, S_, NC_, RP_, XP_>();
+    if constexpr (MODE == MODE_STEP)
+        if (c.few)
+            return c.lx == 32 ? blocks_inst<T, MODE, 0, 32, 4, 4, 4, 1, 0, 1>()
+                              : blocks_inst<T, MODE, 0, 16, 4, 4, 4, 1, 0, 1>();
     if (c.rag == 2) return blocks_inst<T, MODE, 2, 32, 4, 4, 4, 1, 0>();
     if (c.rag) {
 #define PW_OCC_RAG 1
