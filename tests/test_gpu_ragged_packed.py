@@ -75,3 +75,16 @@ def test_packed_rows_in_one_segment(nx, nz, dtype, call):
     assert h.tma_config(step=call == "step")["nseg"] == 1
     for a, b in zip(wide, got):
         assert torch.equal(a[1:-1, 1:-1, 1:nx + 1], b[1:-1, 1:-1, 1:nx + 1])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("nx", [97, 127, 130, 133, 191])
+def test_tiled_steps_equal_widened_grid_bitwise(nx, dtype):
+    """Wider ones, on tiles: every cell of a row's tail, and the images."""
+    ny, nz = 169 if nx < 127 else 129, 130          # above the least size of FP32 steps on tiles
+    wide, got, _, _ = _pair(nx, ny, nz, dtype, 1, "step")
+    for a, b in zip(wide, got):
+        assert torch.equal(a[1:-1, 1:-1, 1:nx + 1], b[1:-1, 1:-1, 1:nx + 1])
+        v = b[1:-1]
+        assert torch.equal(v[:, :, 0], v[:, :, nx]) and torch.equal(v[:, :, nx + 1], v[:, :, 1])
+        assert torch.equal(v[:, 0], v[:, ny]) and torch.equal(v[:, ny + 1], v[:, 1])
