@@ -173,24 +173,31 @@ bool pw::is_device_ptr(const void* p, int device) {
     return a.type == cudaMemoryTypeDevice && a.device == device;
 }
 
-// Tensor map of a field for a box of box_w x box_h elements, from the
-// handle's cache of recently encoded maps.
-static pw_status_t encode_map_box(pw_handle_t h, const void* ptr, int box_w, int box_h, CUtensorMap* out) {
+// The entry of a handle's cache of recently encoded maps for these cells of a
+// field and this box, its map encoded by `encode` (a status) if it is not there.
+template <class Encode>
+static pw_status_t cached_map(pw_handle_t h, const void* ptr, int kind, int box_w, int box_h, CUtensorMap* out,
+                              const Encode& encode) {
     for (auto& c : h->maps)
-        if (c.ptr == ptr && c.kind == MAP_FIELD && c.box_w == box_w && c.box_h == box_h) {
+        if (c.ptr == ptr && c.kind == kind && c.box_w == box_w && c.box_h == box_h) {
             *out = c.map;
             return PW_OK;
         }
+    const pw_status_t st = encode();
+    if (st != PW_OK) return st;
     MapCacheEntry& e = h->maps[h->map_next];
     h->map_next = (h->map_next + 1) % (int)(sizeof(h->maps) / sizeof(h->maps[0]));
-    pw_status_t st = encode_tensor_map_box(h->grid, ptr, box_w, box_h, out);
-    if (st != PW_OK) return st;
     e.ptr = ptr;
-    e.kind = MAP_FIELD;
+    e.kind = kind;
     e.box_w = box_w;
     e.box_h = box_h;
     e.map = *out;
     return PW_OK;
+}
+
+static pw_status_t encode_map_box(pw_handle_t h, const void* ptr, int box_w, int box_h, CUtensorMap* out) {
+    return cached_map(h, ptr, MAP_FIELD, box_w, box_h, out,
+                      [&] { return encode_tensor_map_box(h->grid, ptr, box_w, box_h, out); });
 }
 
 // Tensor map for a launch shape of the single-grid k-march.
@@ -255,11 +262,6 @@ static AdjGeom adj_geom(const pw_grid_t& g, int ox, AdjMode mode) {
 static pw_status_t adj_map(pw_handle_t h, int f, const void* ptr, AdjMode mode, int ox, int box_w, int box_h,
                            CUtensorMap* out) {
     const int kind = MAP_ADJ + 3 * (f < 3 ? 0 : (f < 5 ? 1 : 2)) + (int)mode;
-    for (auto& c : h->maps)
-        if (c.ptr == ptr && c.kind == kind && c.box_w == box_w && c.box_h == box_h) {
-            *out = c.map;
-            return PW_OK;
-        }
     const pw_grid_t& g = h->grid;
     const AdjGeom ge = adj_geom(g, ox, mode);
     // the map's first element: level, row and column with coordinate 0
@@ -269,16 +271,8 @@ static pw_status_t adj_map(pw_handle_t h, int f, const void* ptr, AdjMode mode, 
     const bool whole = mode == ADJ_PERIODIC || (mode == ADJ_PERIODIC_ANY && f < 3);
     const long long rows = whole ? g.ny + 2LL * g.halo : (f < 3 ? g.ny + 2 : g.ny);
     const long long cols = whole ? ox + g.nx + g.halo + 1LL : (f < 3 ? g.nx + 5 : g.nx);
-    pw_status_t st = encode_tensor_map_dims(g, base, {cols, rows, levels}, box_w, box_h, out);
-    if (st != PW_OK) return st;
-    MapCacheEntry& e = h->maps[h->map_next];
-    h->map_next = (h->map_next + 1) % (int)(sizeof(h->maps) / sizeof(h->maps[0]));
-    e.ptr = ptr;
-    e.kind = kind;
-    e.box_w = box_w;
-    e.box_h = box_h;
-    e.map = *out;
-    return PW_OK;
+    return cached_map(h, ptr, kind, box_w, box_h, out,
+                      [&] { return encode_tensor_map_dims(g, base, {cols, rows, levels}, box_w, box_h, out); });
 }
 
 // Every pointer in ps[0..n) is device memory of the handle's GPU (checked
