@@ -415,17 +415,23 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
 // 21.3.  pw_set_kernel(2) refuses such a width as it always has.
 constexpr int kRagMinNx = 32;
 constexpr long long kRagMinCells = 1 << 19, kRagMinStepCells = 1 << 21;
+static bool ragged_on_march(pw_handle_t h, bool step) {
+    const TmaConfig& u = h->tma_user;
+    const pw_grid_t& gr = h->grid;
+    const long long cells = (long long)gr.nx * gr.ny * gr.nz;
+    if (h->kernel_kind != 0 || gr.nx < kRagMinNx || cells < kRagMinCells || u.lx || u.nc || u.ty || u.stages || u.rp)
+        return false;
+    const bool packed = gr.nx <= (gr.dtype == PW_F32 ? kPackedNx : kPackedNx16);
+    if (!packed && step && gr.dtype == PW_F32 && cells < kRagMinStepCells &&
+        10LL * ((gr.nx + 31) / 32 * 32) > 11LL * gr.nx)
+        return false;
+    const int rows = packed ? packed_rows(gr.nx, (int)dtype_size(gr.dtype)).rows : 4;   // the lowest tile's
+    return gr.ny <= (long long)kMaxGridY * rows;
+}
 static pw_status_t march_kernel_choice(pw_handle_t h, bool step, const void* const* bufs, int n, bool* use_tma,
                                        int* ox) {
     const char* why = "";
-    const TmaConfig& u = h->tma_user;
-    const pw_grid_t& gr = h->grid;
-    const bool loose = step && gr.dtype == PW_F32 && gr.nx > kPackedNx && 10LL * ((gr.nx + 31) / 32 * 32) > 11LL * gr.nx;
-    const bool packed = gr.nx <= (gr.dtype == PW_F32 ? kPackedNx : kPackedNx16);
-    const int rows = packed ? packed_rows(gr.nx, (int)dtype_size(gr.dtype)).rows : 4;   // the lowest tile's
-    const bool any_nx = h->kernel_kind == 0 && gr.nx >= kRagMinNx && gr.ny <= (long long)kMaxGridY * rows &&
-                        (long long)gr.nx * gr.ny * gr.nz >= (loose ? kRagMinStepCells : kRagMinCells) &&
-                        !(u.lx || u.nc || u.ty || u.stages || u.rp);
+    const bool any_nx = h->grid.nx % 4 && ragged_on_march(h, step);
     const bool layout_ok = tma_layout_ok(h->grid, ox, &why, any_nx);
     bool ptrs_ok = true;
     for (int a = 0; a < n; ++a) ptrs_ok = ptrs_ok && aligned16(bufs[a]);
@@ -677,7 +683,11 @@ static bool adj_fixed(pw_handle_t h) {
 // kShapeMinCells, and 16 lanes x 4 cells x 8 rows with 3 slots otherwise; k
 // segments (automatic) of >= 4 levels, the count with the lowest estimated
 // time as for the k-march, a segment's start costing 2.5 levels (two planes
-// more than its levels, the priming level).
+// more than its levels, the priming level).  Periodic small grids, (4, 6, 4) / (4,
+// 8, 3) in us: 64x8x4 8.2 / 8.9, 32x32x32 8.9 / 8.6, 64x64x32 8.9 / 8.7, 128x64x30
+// 10.1 / 9.6, 64x64x64 10.3 / 9.4.  The full array has (4, 8, 3) alone, against the
+// gather kernel 8x8x8 7.2 / 20.5, 32x32x16 7.9 / 18.8, 64x64x64 9.8 / 44.6; odd periodic
+// widths 127x64x40 26.8 / 30.6, 33x250x60 35.8 / 48.6.
 static AdjConfig choose_adjoint(pw_handle_t h, AdjMode mode) {
     AdjConfig& cache = h->adj_auto[mode];
     if (cache.na) return cache;
