@@ -330,14 +330,26 @@ constexpr int kPackedNx = 80, kPackedNx16 = 96;
 // shapes and segments over 31 grids (64^3 to 1056 x 1552 x 24): in the mean the
 // choice is within 1 % (FP32 source terms), 2 % (16-bit), 3 to 4 % (steps) of
 // the sweep's best, where counting whole waves of (levels + 2) was 8 % off.
-static double march_cost(const pw_grid_t& gr, const TmaConfig& c, int n, int sms, int bps) {
+// FP32 steps, after a sweep over 135 grids from 2e4 to 4e7 cells: 0.3 of a wave
+// more where the fields exceed L2 (kL2Cells), 0.4 for grids at most 64 columns wide:
+// the time in which the first and last CTAs leave the memory idle.  Without it one
+// wave of whole columns looks too cheap there (652 x 449 x 55: one segment 101 us, four
+// 86, 8-lane tiles in seven 80; 56 x 1088 x 84: five 48, eight 42).  The choice is then
+// within 1.2 % of the sweep's best in the mean.
+constexpr long long kL2Cells = 6000000;   // 24 bytes each: a little more than L2
+static long long march_tiles(const pw_grid_t& gr, const TmaConfig& c) {
     const int rows = c.rag == 2 ? packed_rows(gr.nx, (int)dtype_size(gr.dtype)).rows : c.ty;
-    const long long tiles = (c.rag == 2 ? 1LL : (gr.nx + c.nc * c.lx - 1) / (c.nc * c.lx)) * ((gr.ny + rows - 1) / rows);
-    const long long ctas = tiles * n, slots = (long long)sms * bps;
+    return (c.rag == 2 ? 1LL : (gr.nx + c.nc * c.lx - 1) / (c.nc * c.lx)) * ((gr.ny + rows - 1) / rows);
+}
+static double march_cost(const pw_grid_t& gr, const TmaConfig& c, bool step, int n, int sms, int bps) {
+    const long long ctas = march_tiles(gr, c) * n, slots = (long long)sms * bps;
     const long long full = ctas / slots, rem = ctas - full * slots;
     const double w = c.xp ? 0.45 : 0.7;
+    double out = 0.0;
+    if (step && gr.dtype == PW_F32 && !c.rag)
+        out = gr.nx <= 64 ? 0.4 : ((long long)gr.nx * gr.ny * gr.nz > kL2Cells ? 0.3 : 0.0);
     const double last = rem ? w + (1.0 - w) * (double)((rem + sms - 1) / sms) / bps : 0.0;
-    return ((gr.nz + n - 1) / n + (c.xp ? 0.8 : 1.6)) * ((double)full + last) * bps * (c.nc * c.lx) * c.ty;
+    return ((gr.nz + n - 1) / n + (c.xp ? 0.8 : 1.6)) * ((double)full + last + out) * bps * (c.nc * c.lx) * c.ty;
 }
 
 static TmaConfig choose_tma(pw_handle_t h, bool step) {
@@ -345,7 +357,7 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
     if (cache.ty) return cache;
     const TmaConfig& u = h->tma_user;
     const pw_grid_t& gr = h->grid;
-    TmaConfig cand[3];
+    TmaConfig cand[4];
     int nc = 0;
     auto add = [&](int lx, int cells, int ty, int xp, int rp) {
         TmaConfig c{lx, ty, 4, 1, cells};
@@ -365,6 +377,8 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
             add(16, 4, 4, 0, 1);
         } else if (!half) {
             add(32, 4, 4, 0, 1);
+            if (step && gr.nx % 4 == 0) cand[0].few = 1;
+            if (cand[0].few && more) add(32, 4, 4, 0, 1);
             if (more) add(16, 4, 8, 0, 1);
             if (more) add(8, 4, 16, 0, 1);
         } else if (!step || gr.nx % 8 == 0) {
@@ -375,9 +389,8 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
             if (more) add(16, 4, 8, 1, 1);
         }
         for (int q = 0; q < nc; ++q) cand[q].rag = gr.nx % 4 ? (packed ? 2 : 1) : 0;
-        const long long cells = (long long)gr.nx * gr.ny * gr.nz;   // (see tma_min_blocks)
-        if (step && gr.nx % 4 == 0 && !cand[0].xp)
-            cand[0].few = gr.nx > 64 ? cells <= (1 << 20) : gr.nx < 64 && cells < (1 << 17);
+        if (step && gr.nx % 4 == 0 && gr.nx < 64)   // (see tma_min_blocks)
+            cand[0].few = (long long)gr.nx * gr.ny * gr.nz < (1 << 17);
     }
     TmaConfig best = cand[0];
     double lowest = 0.0;
@@ -387,7 +400,8 @@ static TmaConfig choose_tma(pw_handle_t h, bool step) {
         if (bps < 1) bps = 1;
         const int lo = u.nseg ? u.nseg : 1, hi = u.nseg ? u.nseg : std::max(1, gr.nz / 2);
         for (c.nseg = lo; c.nseg <= hi; ++c.nseg) {
-            const double cost = march_cost(gr, c, c.nseg, h->num_sms, bps);
+            if (c.few && nc > 1 && march_tiles(gr, c) * c.nseg > (long long)h->num_sms * bps) break;
+            const double cost = march_cost(gr, c, step, c.nseg, h->num_sms, bps);
             if (lowest > 0.0 && !(cost < 0.985 * lowest)) continue;   // narrower or more segments only for a gain
             lowest = cost;
             best = c;

@@ -915,12 +915,13 @@ struct TmaLayout {
 // BF16 against the compiler's 210 registers, as more CTAs per SM hide more
 // latency; 128 spills and 200 leaves 2 CTAs per SM, both slower).
 //
-// FEW: the scalar step of a grid of few cells, which waits for a level's latency
-// and has no use for a fifth CTA per SM: the compiler's registers on 32 lanes,
-// one test for the images (store_field) on 16.  us a step, capped at PW_STEP_REGS
-// with single predicated stores / FEW: 120 x 64 x
-// 17 5.2 / 4.8, 88 x 18 x 43 5.3 / 4.9, 128 x 128 x 64 8.4 / 8.2 (256 x 128 x 64 13.2 /
-// 13.5: not above 2^20 cells); 32 x 69 x 25 5.1 / 4.9, 52 x 52 x 43 4.9 / 4.8 (44 x 119
+// FEW: the scalar step of few CTAs, which waits for a level's latency and has no
+// use for a fifth CTA per SM: the compiler's registers on 32 lanes, one test for
+// the images (store_field) on 16.  us a step, capped at PW_STEP_REGS with single
+// predicated stores / FEW: 120 x 64 x 17 5.2 / 4.8, 88 x 18 x 43 5.3 / 4.9, in one wave
+// 592 x 89 x 38 15.5 / 13.6, 1472 x 20 x 74 15.0 / 13.8, 256 x 256 x 64 25.5 / 24.2 (in two
+// 512 x 512 x 64 76 / 85: on 32 lanes for grids below 2^18 cells and launches of one
+// wave of four CTAs per SM); 32 x 69 x 25 5.1 / 4.9, 52 x 52 x 43 4.9 / 4.8 (44 x 119
 // x 33 5.2 / 5.5, 64 columns 0.1 slower: not from 2^17 cells, not at 64 columns).
 // The cap is for FP32 storage: 16-bit scalar steps, at most 64 columns wide, take
 // 4.74 us at 64^3 without it and 4.95 with it, 32 x 69 x 25 5.37 and 5.58.

@@ -1,8 +1,9 @@
-"""Fused steps of grids of few cells run an instance of their own.
+"""Fused steps of few CTAs run an instance of their own.
 
 It gives the bits of the instance larger grids take (forced here by fixing the
 shape), halo images included, on both sides of the rule's limits: 2^17 cells and
-64 columns for 16 lanes per row, 2^20 cells for 32."""
+64 columns for 16 lanes per row; 2^18 cells, and above that one wave of CTAs (608 on
+152 SMs), for 32."""
 import pytest
 import torch
 
@@ -15,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("dtype,shape", [("f32", s) for s in (
     (4, 1, 3), (60, 1, 12), (60, 5, 3), (52, 52, 43), (60, 84, 26), (60, 85, 26), (64, 30, 20),     # 131040, 132600 cells
-    (68, 1, 3), (68, 9, 12), (120, 64, 17), (132, 7, 70), (256, 64, 64), (256, 65, 64))] + [
+    (68, 1, 3), (68, 9, 12), (120, 64, 17), (132, 7, 70), (256, 32, 32), (256, 33, 32), (592, 89, 38), (256, 256, 64))] + [
     ("bf16", (60, 5, 7)), ("bf16", (32, 69, 25)), ("f16", (60, 84, 26))])
 def test_few_cells_give_the_same_bits(dtype, shape):
     nx, ny, nz = shape
